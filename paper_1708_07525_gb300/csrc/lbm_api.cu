@@ -156,6 +156,10 @@ const char* check_params(const lbm_params& P) {
 
 }  // namespace
 
+// d_out: Nu/Sh of the side walls at 0, residual maxima at 8, Nu/Sh of bottom and top at
+// 20, scratch of the Nu/Sh pass at 64.
+constexpr int OUT_SCRATCH = 64, OUT_DOUBLES = OUT_SCRATCH + NUSH_SCRATCH;
+
 struct lbm_ctx {
     lbm_params P;
     int prec = LBM_F64, layout = LBM_AB_PULL;
@@ -163,7 +167,7 @@ struct lbm_ctx {
     size_t esz = 8, rsz = 8;
     void* buf[2] = {nullptr, nullptr};
     void* hist = nullptr;
-    double* d_out = nullptr;        // 16 doubles: Nu/Sh and residual results
+    double* d_out = nullptr;        // OUT_DOUBLES: Nu/Sh and residual results, Nu/Sh partial sums
     double* d_fields = nullptr;     // lazily allocated [5][h][w] read-out window
     size_t fields_cap = 0;          // nodes d_fields holds
     void* d_snap = nullptr;         // lazily allocated [4][ny][nx] in the compute precision
@@ -662,7 +666,7 @@ lbm_status create_core(const lbm_params* params, const lbm_options* opt, int sla
     c->buf[0] = c->dalloc(c->state_bytes());
     if (c->layout == LBM_AB_PULL) c->buf[1] = c->dalloc(c->state_bytes());
     c->hist = c->dalloc(c->hist_bytes());
-    c->d_out = (double*)c->dalloc(64 * sizeof(double));
+    c->d_out = (double*)c->dalloc(OUT_DOUBLES * sizeof(double));
     if (O.eps_field || O.K_field) {
         if (c->P.model_a) {
             lbm_status s = c->fail(LBM_ERR_INVALID, "lbm_create: porous fields are not supported with model_a");
@@ -724,6 +728,7 @@ lbm_status create_core(const lbm_params* params, const lbm_options* opt, int sla
     cudaMemsetAsync(c->buf[0], 0, c->state_bytes(), c->stream);
     if (c->buf[1]) cudaMemsetAsync(c->buf[1], 0, c->state_bytes(), c->stream);
     cudaMemsetAsync(c->hist, 0, c->hist_bytes(), c->stream);
+    cudaMemsetAsync(c->d_out, 0, OUT_DOUBLES * sizeof(double), c->stream);   // the block count of the Nu/Sh pass
 
     if ((O.T_init == nullptr) != (O.C_init == nullptr)) {
         lbm_status s = c->fail(LBM_ERR_INVALID, "lbm_create: give both T_init and C_init");
@@ -902,10 +907,10 @@ lbm_status lbm_nusselt_sherwood(lbm_ctx* c, double out[4]) {
     W.L = c->P.nee ? c->P.nx - 1.0 : (double)c->P.nx;
     const int mode = c->read_mode();
     const void* b = cur_buf(c);
-    cudaError_t e = LBM_DISPATCH(c, launch_nush<double>(b, c->G, c->cd, mode, W, c->d_out, c->stream),
-                                 launch_nush<float>(b, c->G, c->cf, mode, W, c->d_out, c->stream),
-                                 launch_nush<__nv_bfloat16>(b, c->G, c->cf, mode, W, c->d_out, c->stream),
-                                 launch_nush<__half>(b, c->G, c->cf, mode, W, c->d_out, c->stream));
+    cudaError_t e = LBM_DISPATCH(c, launch_nush<double>(b, c->G, c->cd, mode, W, c->d_out + OUT_SCRATCH, c->d_out, c->stream),
+                                 launch_nush<float>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, c->d_out, c->stream),
+                                 launch_nush<__nv_bfloat16>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, c->d_out, c->stream),
+                                 launch_nush<__half>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, c->d_out, c->stream));
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(out, c->d_out, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -937,10 +942,10 @@ lbm_status lbm_nusselt_sherwood_tb(lbm_ctx* c, double out[4]) {
     W.L = c->P.nee ? c->P.ny - 1.0 : (double)c->P.ny;
     const int mode = c->read_mode();
     const void* b = cur_buf(c);
-    cudaError_t e = LBM_DISPATCH(c, launch_nush_tb<double>(b, c->G, c->cd, mode, W, c->d_out + 20, c->stream),
-                                 launch_nush_tb<float>(b, c->G, c->cf, mode, W, c->d_out + 20, c->stream),
-                                 launch_nush_tb<__nv_bfloat16>(b, c->G, c->cf, mode, W, c->d_out + 20, c->stream),
-                                 launch_nush_tb<__half>(b, c->G, c->cf, mode, W, c->d_out + 20, c->stream));
+    cudaError_t e = LBM_DISPATCH(c, launch_nush_tb<double>(b, c->G, c->cd, mode, W, c->d_out + OUT_SCRATCH, c->d_out + 20, c->stream),
+                                 launch_nush_tb<float>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, c->d_out + 20, c->stream),
+                                 launch_nush_tb<__nv_bfloat16>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, c->d_out + 20, c->stream),
+                                 launch_nush_tb<__half>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, c->d_out + 20, c->stream));
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(out, c->d_out + 20, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -961,7 +966,7 @@ lbm_status residual_maxima(lbm_ctx* c, const char* who, double h[9]) {
     const size_t n = c->nodes();
     if (!c->d_snap) {
         c->d_snap = c->dalloc(4 * n * c->rsz);
-        c->d_partial = (double*)c->dalloc((size_t)RES_SLOTS * 9 * sizeof(double));
+        c->d_partial = (double*)c->dalloc(RES_SCRATCH * sizeof(double));
         if (!c->d_snap || !c->d_partial) return c->fail(LBM_ERR_NOMEM, "%s: no device memory", who);
     }
     const int mode = c->read_mode();
@@ -1235,10 +1240,10 @@ void lbm_destroy(lbm_ctx* c) {
     c->dfree(c->buf[0], c->state_bytes());
     c->dfree(c->buf[1], c->state_bytes());
     c->dfree(c->hist, c->hist_bytes());
-    c->dfree(c->d_out, 64 * sizeof(double));
+    c->dfree(c->d_out, OUT_DOUBLES * sizeof(double));
     c->dfree(c->d_fields, 5 * c->fields_cap * sizeof(double));
     c->dfree(c->d_snap, 4 * c->nodes() * c->rsz);
-    c->dfree(c->d_partial, (size_t)RES_SLOTS * 9 * sizeof(double));
+    c->dfree(c->d_partial, RES_SCRATCH * sizeof(double));
     c->dfree(c->d_stage, 2 * c->nodes() * sizeof(double));
     c->dfree(c->poro, 2 * c->G.plane * c->rsz);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);

@@ -260,73 +260,63 @@ batch_residual_fold_kernel(const BatchInst<R>* __restrict__ table, const int* __
     }
 }
 
-// Nu / Sh of every cavity (Eq. 38): block k reduces cavity k's wall columns.
+// Nu / Sh of every cavity (Eq. 38): block (k, s) reduces the left (s = 0) or right wall of
+// cavity k, with the stencils of nush_kernel.  Both walls in one block took 232-250
+// registers and 22 us for 24 cavities of up to 256^2; a wall is half the serial work.
 template <typename S, bool AA>
 __global__ void __launch_bounds__(BATCH_THREADS)
 batch_nush_kernel(const BatchInst<typename Real<S>::type>* __restrict__ table,
                   const WallSpec* __restrict__ walls, int parity, double* __restrict__ out) {
     using R = typename Real<S>::type;
-    const int k = blockIdx.x;
+    const int k = blockIdx.x, far = blockIdx.y;
     __shared__ BatchInst<R> I;
     load_inst(table, k, I);
     __syncthreads();
-    double acc[4] = {0, 0, 0, 0};
-    const WallSpec W = walls[k];
+    double aT = 0, aC = 0;
+    const WallSpec& W = walls[k];
     if (I.active) {
         const int mode = batch_mode(I, parity, AA);
         const S* buf = (const S*)batch_cur(I, parity, AA);
         const Geom G = I.G;
-        if (W.nee) {
-            // nodes on the walls: the node stencil and the trapezoidal mean of nush_kernel
-            for (int j = threadIdx.x; j < G.ny; j += blockDim.x) {
-                R f[9], g[5], h[5];
-                double T[6], C[6];
-                const int cols[6] = {0, 1, 2, G.nx - 3, G.nx - 2, G.nx - 1};
+        for (int j = threadIdx.x; j < G.ny; j += blockDim.x) {
+            double T[3], C[3];
 #pragma unroll
-                for (int q = 0; q < 6; ++q) {
-                    gather<false>(mode, buf, G, cols[q], j, I.c, f, g, h);
-                    const R sg = ((g[0] + g[1]) + (g[2] + g[3])) + g[4];
-                    const R sh = ((h[0] + h[1]) + (h[2] + h[3])) + h[4];
-                    T[q] = W.T0 + (double)(sg * I.c.inv_sigma);
-                    C[q] = W.C0 + (double)(sh * I.c.inv_eps);
+            for (int q = 0; q < 3; ++q) {
+                if (q == 2 && !W.nee) {
+                    T[2] = C[2] = 0;
+                    continue;
                 }
-                const double wj = (j == 0 || j == G.ny - 1) ? 0.5 : 1.0;
-                acc[0] += wj * -W.L * (-3.0 * T[0] + 4.0 * T[1] - T[2]) / 2.0 / W.dT;
-                acc[1] += wj * -W.L * (-3.0 * C[0] + 4.0 * C[1] - C[2]) / 2.0 / W.dC;
-                acc[2] += wj * -W.L * (3.0 * T[5] - 4.0 * T[4] + T[3]) / 2.0 / W.dT;
-                acc[3] += wj * -W.L * (3.0 * C[5] - 4.0 * C[4] + C[3]) / 2.0 / W.dC;
-            }
-        }
-        for (int j = threadIdx.x; j < G.ny && !W.nee; j += blockDim.x) {
-            R f[9], g[5], h[5];
-            double T[4], C[4];
-            const int cols[4] = {0, 1, G.nx - 2, G.nx - 1};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                gather<false>(mode, buf, G, cols[q], j, I.c, f, g, h);
+                R f[9], g[5], h[5];
+                gather<false>(mode, buf, G, far ? G.nx - 1 - q : q, j, I.c, f, g, h);
                 const R sg = ((g[0] + g[1]) + (g[2] + g[3])) + g[4];
                 const R sh = ((h[0] + h[1]) + (h[2] + h[3])) + h[4];
                 T[q] = W.T0 + (double)(sg * I.c.inv_sigma);
                 C[q] = W.C0 + (double)(sh * I.c.inv_eps);
             }
-            acc[0] += -W.L * (-8.0 * W.Tw[0] + 9.0 * T[0] - T[1]) / 3.0 / W.dT;
-            acc[1] += -W.L * (-8.0 * W.Cw[0] + 9.0 * C[0] - C[1]) / 3.0 / W.dC;
-            acc[2] += -W.L * (8.0 * W.Tw[1] - 9.0 * T[3] + T[2]) / 3.0 / W.dT;
-            acc[3] += -W.L * (8.0 * W.Cw[1] - 9.0 * C[3] + C[2]) / 3.0 / W.dC;
+            if (W.nee) {
+                const double w = (j == 0 || j == G.ny - 1) ? 0.5 : 1.0;
+                aT += w * ((-3.0 * T[0] + 4.0 * T[1] - T[2]) / 2.0);
+                aC += w * ((-3.0 * C[0] + 4.0 * C[1] - C[2]) / 2.0);
+            } else {
+                aT += (-8.0 * W.Tw[far] + 9.0 * T[0] - T[1]) / 3.0;
+                aC += (-8.0 * W.Cw[far] + 9.0 * C[0] - C[1]) / 3.0;
+            }
         }
     }
-    __shared__ double red[BATCH_THREADS / 32][4];
+    __shared__ double red[BATCH_THREADS / 32][2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const double v = warp_sum(acc[q]);
-        if (lane == 0) red[warp][q] = v;
+    aT = warp_sum(aT);
+    aC = warp_sum(aC);
+    if (lane == 0) {
+        red[warp][0] = aT;
+        red[warp][1] = aC;
     }
     __syncthreads();
-    if (threadIdx.x < 4) {
+    if (threadIdx.x < 2) {
         double s = 0;
         for (int w = 0; w < BATCH_THREADS / 32; ++w) s += red[w][threadIdx.x];
-        out[(size_t)k * 4 + threadIdx.x] = I.active ? s / (W.nee ? I.G.ny - 1.0 : (double)I.G.ny) : 0.0;
+        const double scale = W.L / (threadIdx.x ? W.dC : W.dT) / (W.nee ? I.G.ny - 1.0 : (double)I.G.ny);
+        out[(size_t)k * 4 + 2 * far + threadIdx.x] = I.active ? s * (far ? scale : -scale) : 0.0;
     }
 }
 

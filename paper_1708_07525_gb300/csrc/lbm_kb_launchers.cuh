@@ -57,9 +57,9 @@ cudaError_t launch_batch_nush(const BatchInst<float>* table, const WallSpec* wal
                               int parity, bool aa, double* out, cudaStream_t st) {
     if (n_inst <= 0) return cudaSuccess;
     if (aa)
-        batch_nush_kernel<S, true><<<n_inst, BATCH_THREADS, 0, st>>>(table, walls, parity, out);
+        batch_nush_kernel<S, true><<<dim3((unsigned)n_inst, 2), BATCH_THREADS, 0, st>>>(table, walls, parity, out);
     else
-        batch_nush_kernel<S, false><<<n_inst, BATCH_THREADS, 0, st>>>(table, walls, parity, out);
+        batch_nush_kernel<S, false><<<dim3((unsigned)n_inst, 2), BATCH_THREADS, 0, st>>>(table, walls, parity, out);
     return cudaGetLastError();
 }
 

@@ -839,144 +839,107 @@ __device__ __forceinline__ float warp_max(float v) {
     return v;
 }
 
-// Mean Nu / Sh on the left and right walls (Eq. 38), one block, FP64 sums with a
-// fixed reduction order (deterministic).  out = {Nu_L, Sh_L, Nu_R, Sh_R}.
-template <typename S>
+// Mean Nu / Sh on a pair of opposite walls (Eq. 38), FP64 sums with a fixed reduction
+// order (deterministic).  LR = true: the left and right walls, out = {Nu_L, Sh_L, Nu_R,
+// Sh_R}; false: bottom and top (W.Tw / W.Cw = {bottom, top}), out = {Nu_B, Sh_B, Nu_T, Sh_T}.
+// Grid (nush_blocks(G, LR), 2): block (b, s) takes the line positions b * NUSH_THREADS + t, plus
+// multiples of gridDim.x * NUSH_THREADS, of wall s, and the block that finishes last adds
+// the partial sums in block order.  `part` holds 2 * NUSH_MAX_BLOCKS pairs of doubles,
+// *done counts finished blocks (0 before the launch; the last block puts it back).
+// Bound by latency and by the FP64 pipe (half a lane per clock and SM sub-partition): one
+// block of 512 threads with both walls in each thread took 24 us at 256^2, 56 us at
+// 1024^2 and 90 us at 2048^2 (FP32); spread over the SMs it is one node pair's chain.
+template <typename S, bool LR>
 __global__ void __launch_bounds__(NUSH_THREADS)
 nush_kernel(const S* __restrict__ buf, Geom G, Coef<typename Real<S>::type> c, int mode,
-            WallSpec W, double* __restrict__ out) {
+            WallSpec W, double* __restrict__ part, unsigned* __restrict__ done,
+            double* __restrict__ out) {
     using R = typename Real<S>::type;
-    double acc[4] = {0, 0, 0, 0};
-    if (W.nee) {
-        // nodes on the walls: dPhi/dx|wall = (-3 Phi_0 + 4 Phi_1 - Phi_2) / 2, mirrored on
-        // the right; trapezoidal mean over the ny - 1 spacings
-        for (int j = threadIdx.x; j < G.ny; j += blockDim.x) {
-            R f[9], g[5], h[5];
-            double T[6], C[6];
-            const int cols[6] = {0, 1, 2, G.nx - 3, G.nx - 2, G.nx - 1};
+    const int far = blockIdx.y;                          // 0: left / bottom, 1: right / top
+    const int across = LR ? G.nx : G.ny;                 // nodes from wall to wall
+    const int j0 = LR ? G.jb : 0, j1 = LR ? G.je : G.nx;   // positions along the wall
+    double aT = 0, aC = 0;
+    for (int j = j0 + (int)(blockIdx.x * blockDim.x + threadIdx.x); j < j1; j += gridDim.x * blockDim.x) {
+        double T[3], C[3];
+        // the wall's three (nodes on the walls) or two (halfway walls) nearest nodes
 #pragma unroll
-            for (int k = 0; k < 6; ++k) {
-                gather<false>(mode, buf, G, cols[k], j, c, f, g, h);
-                const R sg = ((g[0] + g[1]) + (g[2] + g[3])) + g[4];
-                const R sh = ((h[0] + h[1]) + (h[2] + h[3])) + h[4];
-                const R ie = c.poro ? R(1) / c.poro[(size_t)j * G.pitch + cols[k]] : c.inv_eps;
-                T[k] = W.T0 + (double)(sg * c.inv_sigma);
-                C[k] = W.C0 + (double)(sh * ie);
+        for (int k = 0; k < 3; ++k) {
+            if (k == 2 && !W.nee) {
+                T[2] = C[2] = 0;
+                continue;
             }
-            const double wj = (j == 0 || j == G.ny - 1) ? 0.5 : 1.0;
-            acc[0] += wj * -W.L * (-3.0 * T[0] + 4.0 * T[1] - T[2]) / 2.0 / W.dT;
-            acc[1] += wj * -W.L * (-3.0 * C[0] + 4.0 * C[1] - C[2]) / 2.0 / W.dC;
-            acc[2] += wj * -W.L * (3.0 * T[5] - 4.0 * T[4] + T[3]) / 2.0 / W.dT;
-            acc[3] += wj * -W.L * (3.0 * C[5] - 4.0 * C[4] + C[3]) / 2.0 / W.dC;
-        }
-    }
-    for (int j = G.jb + threadIdx.x; j < G.je && !W.nee; j += blockDim.x) {
-        R f[9], g[5], h[5];
-        double T[4], C[4];
-        const int cols[4] = {0, 1, G.nx - 2, G.nx - 1};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            gather<false>(mode, buf, G, cols[k], j, c, f, g, h);
+            const int d = far ? across - 1 - k : k;
+            const int i = LR ? d : j, jj = LR ? j : d;
+            R f[9], g[5], h[5];
+            gather<false>(mode, buf, G, i, jj, c, f, g, h);
             const R sg = ((g[0] + g[1]) + (g[2] + g[3])) + g[4];
             const R sh = ((h[0] + h[1]) + (h[2] + h[3])) + h[4];
-            const R ie = c.poro ? R(1) / c.poro[(size_t)j * G.pitch + cols[k]] : c.inv_eps;
+            const R ie = c.poro ? R(1) / c.poro[(size_t)jj * G.pitch + i] : c.inv_eps;
             T[k] = W.T0 + (double)(sg * c.inv_sigma);
             C[k] = W.C0 + (double)(sh * ie);
         }
-        // dPhi/dx at the wall: (-8 Phi_w + 9 Phi_0 - Phi_1) / 3, mirrored on the right
-        acc[0] += -W.L * (-8.0 * W.Tw[0] + 9.0 * T[0] - T[1]) / 3.0 / W.dT;
-        acc[1] += -W.L * (-8.0 * W.Cw[0] + 9.0 * C[0] - C[1]) / 3.0 / W.dC;
-        acc[2] += -W.L * (8.0 * W.Tw[1] - 9.0 * T[3] + T[2]) / 3.0 / W.dT;
-        acc[3] += -W.L * (8.0 * W.Cw[1] - 9.0 * C[3] + C[2]) / 3.0 / W.dC;
-    }
-    __shared__ double red[NUSH_THREADS / 32][4];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const double v = warp_sum(acc[k]);
-        if (lane == 0) red[warp][k] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 4) {
-        double s = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w][threadIdx.x];
-        out[threadIdx.x] = s / (W.nee ? G.ny - 1.0 : (double)step_rows(G));
-    }
-}
-
-// Mean Nu / Sh on the bottom and top walls, one block, FP64, fixed reduction order.
-// W.Tw / W.Cw = {bottom, top}; out = {Nu_B, Sh_B, Nu_T, Sh_T}.
-template <typename S>
-__global__ void __launch_bounds__(NUSH_THREADS)
-nush_tb_kernel(const S* __restrict__ buf, Geom G, Coef<typename Real<S>::type> c, int mode,
-               WallSpec W, double* __restrict__ out) {
-    using R = typename Real<S>::type;
-    double acc[4] = {0, 0, 0, 0};
-    if (W.nee) {
-        // as on the left / right walls, transposed (node stencil, trapezoidal mean over x)
-        for (int i = threadIdx.x; i < G.nx; i += blockDim.x) {
-            R f[9], g[5], h[5];
-            double T[6], C[6];
-            const int rows[6] = {0, 1, 2, G.ny - 3, G.ny - 2, G.ny - 1};
-#pragma unroll
-            for (int k = 0; k < 6; ++k) {
-                gather<false>(mode, buf, G, i, rows[k], c, f, g, h);
-                const R sg = ((g[0] + g[1]) + (g[2] + g[3])) + g[4];
-                const R sh = ((h[0] + h[1]) + (h[2] + h[3])) + h[4];
-                const R ie = c.poro ? R(1) / c.poro[(size_t)rows[k] * G.pitch + i] : c.inv_eps;
-                T[k] = W.T0 + (double)(sg * c.inv_sigma);
-                C[k] = W.C0 + (double)(sh * ie);
-            }
-            const double wi = (i == 0 || i == G.nx - 1) ? 0.5 : 1.0;
-            acc[0] += wi * W.L * (-3.0 * T[0] + 4.0 * T[1] - T[2]) / 2.0 / W.dT;
-            acc[1] += wi * W.L * (-3.0 * C[0] + 4.0 * C[1] - C[2]) / 2.0 / W.dC;
-            acc[2] += wi * W.L * (3.0 * T[5] - 4.0 * T[4] + T[3]) / 2.0 / W.dT;
-            acc[3] += wi * W.L * (3.0 * C[5] - 4.0 * C[4] + C[3]) / 2.0 / W.dC;
+        // inward gradient at the wall: nodes on the walls (-3 Phi_0 + 4 Phi_1 - Phi_2) / 2,
+        // trapezoidal mean over the spacings along the wall; halfway walls
+        // (-8 Phi_w + 9 Phi_0 - Phi_1) / 3
+        if (W.nee) {
+            const double w = (j == j0 || j == j1 - 1) ? 0.5 : 1.0;
+            aT += w * ((-3.0 * T[0] + 4.0 * T[1] - T[2]) / 2.0);
+            aC += w * ((-3.0 * C[0] + 4.0 * C[1] - C[2]) / 2.0);
+        } else {
+            aT += (-8.0 * W.Tw[far] + 9.0 * T[0] - T[1]) / 3.0;
+            aC += (-8.0 * W.Cw[far] + 9.0 * C[0] - C[1]) / 3.0;
         }
     }
-    for (int i = threadIdx.x; i < G.nx && !W.nee; i += blockDim.x) {
-        R f[9], g[5], h[5];
-        double T[4], C[4];
-        const int rows[4] = {0, 1, G.ny - 2, G.ny - 1};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            gather<false>(mode, buf, G, i, rows[k], c, f, g, h);
-            const R sg = ((g[0] + g[1]) + (g[2] + g[3])) + g[4];
-            const R sh = ((h[0] + h[1]) + (h[2] + h[3])) + h[4];
-            const R ie = c.poro ? R(1) / c.poro[(size_t)rows[k] * G.pitch + i] : c.inv_eps;
-            T[k] = W.T0 + (double)(sg * c.inv_sigma);
-            C[k] = W.C0 + (double)(sh * ie);
-        }
-        // dPhi/dy at the wall through the wall value and the first two rows
-        acc[0] += W.L * (-8.0 * W.Tw[0] + 9.0 * T[0] - T[1]) / 3.0 / W.dT;
-        acc[1] += W.L * (-8.0 * W.Cw[0] + 9.0 * C[0] - C[1]) / 3.0 / W.dC;
-        acc[2] += W.L * (8.0 * W.Tw[1] - 9.0 * T[3] + T[2]) / 3.0 / W.dT;
-        acc[3] += W.L * (8.0 * W.Cw[1] - 9.0 * C[3] + C[2]) / 3.0 / W.dC;
-    }
-    __shared__ double red[NUSH_THREADS / 32][4];
+    __shared__ double red[NUSH_THREADS / 32][2];
+    __shared__ bool last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const double v = warp_sum(acc[k]);
-        if (lane == 0) red[warp][k] = v;
+    aT = warp_sum(aT);
+    aC = warp_sum(aC);
+    if (lane == 0) {
+        red[warp][0] = aT;
+        red[warp][1] = aC;
     }
     __syncthreads();
-    if (threadIdx.x < 4) {
-        double s = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w][threadIdx.x];
-        out[threadIdx.x] = s / (W.nee ? G.nx - 1.0 : (double)G.nx);
+    if (threadIdx.x == 0) {
+        double* p = part + 2 * ((size_t)far * NUSH_MAX_BLOCKS + blockIdx.x);
+        for (int k = 0; k < 2; ++k) {
+            double v = 0;
+            for (int w = 0; w < NUSH_THREADS / 32; ++w) v += red[w][k];
+            p[k] = v;
+        }
+        __threadfence();                                 // the partial before the count
+        last = atomicAdd(done, 1u) == gridDim.x * gridDim.y - 1;
     }
+    __syncthreads();
+    if (!last) return;
+    if (threadIdx.x < 4) {
+        __threadfence();                                 // the count before the partials
+        const int side = threadIdx.x >> 1, k = threadIdx.x & 1;
+        const volatile double* p = part + 2 * (size_t)side * NUSH_MAX_BLOCKS + k;
+        double v = 0;
+        for (int b = 0; b < (int)gridDim.x; ++b) v += p[2 * b];
+        // dPhi/dn inward at the near wall is +dPhi/dx there and -dPhi/dx at the far wall;
+        // Nu = -L dPhi/dx / dPhi with dPhi = near - far wall (left - right), and for the
+        // bottom / top pair L dPhi/dy over top - bottom
+        const double scale = W.L / (k ? W.dC : W.dT) / (W.nee ? (j1 - j0) - 1.0 : (double)(j1 - j0));
+        out[threadIdx.x] = v * ((side == 0) == LR ? -scale : scale);
+    }
+    if (threadIdx.x == 0) *done = 0;
 }
 
-// Residual pass 1: per node phi = (u_x, u_y, T - T0, C - C0) at the current level
+// Residual: per node phi = (u_x, u_y, T - T0, C - C0) at the current level
 // in the compute precision R (the deviations make the difference of two close
 // values exact); snap (element type P) is replaced by phi.  Each block reduces the
 // maxima of |phi - snap|, of |(u_x, u_y, T, C)| and a non-finite flag, and folds
-// them into slot (block index mod nslots) of slots[nslots][9] with an integer
+// them into slot (block index mod RES_SLOTS) of slots[RES_SLOTS][9] with an integer
 // atomicMax on the FP64 bit patterns (all values are >= 0, whose bit patterns
-// order as the values do); the slots must be zero before the launch.  Block
-// (bx, by) takes the 256-column tiles bx, bx + gridDim.x, ... of the rows by,
-// by + gridDim.y, ...; with the grid of residual_grid() that is one node per thread.
+// order as the values do); the block that finishes last folds the slots into out[9].
+// Slots and the block count behind them (slots[RES_SLOTS * 9]) must be zero before the
+// launch.  Block (bx, by) takes the 256-column tiles bx, bx + gridDim.x, ... of the rows
+// by, by + gridDim.y, ...; with the grid of residual_grid() that is one node per thread.
+// Maxima of FP64 values go through their bit patterns too: the FP64 pipe is the
+// scarce one.  A launch of its own that folded 4096 slots with FP64 maxima took 24 us;
+// 64 slots folded by integer maxima in the last block leave the pass itself.
 // Blocks per SM the residual pass is compiled for: its general gather with the wall rules
 // takes 90 registers left alone (2 blocks of 256 threads per SM, a quarter of the warp
 // slots, for a pass that is all loads).  GB300, 4096^2 FP32 two-buffer, ms per residual
@@ -990,12 +953,35 @@ constexpr int res_min_blocks() {
     return sizeof(typename Real<S>::type) == 8 ? 1 : (MODE == GATHER_NEE_AB ? 3 : LBM_RES_MIN_BLOCKS);
 }
 
+// A non-negative value as bits that order as the values do (NaN above all).
+__device__ __forceinline__ unsigned long long ordered_bits(double x) {
+    return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+}
+__device__ __forceinline__ unsigned ordered_bits(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
+template <typename R> struct Bits { using type = unsigned; };
+template <> struct Bits<double> { using type = unsigned long long; };
+__device__ __forceinline__ double value_of(unsigned long long b) { return __longlong_as_double((long long)b); }
+__device__ __forceinline__ double value_of(unsigned b) { return (double)__uint_as_float(b); }
+template <typename B>
+__device__ __forceinline__ B max_bits(B a, B b) { return a > b ? a : b; }
+__device__ __forceinline__ unsigned warp_max_bits(unsigned v) { return __reduce_max_sync(0xffffffffu, v); }
+__device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max_bits(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+// Whether ordered bits are those of an infinity or a NaN.
+__device__ __forceinline__ bool bits_bad(unsigned b) { return b >= 0x7F800000u; }
+__device__ __forceinline__ bool bits_bad(unsigned long long b) { return b >= 0x7FF0000000000000ull; }
+
 template <typename S, bool EXT, typename P, int MODE>
 __global__ void __launch_bounds__(RES_THREADS, res_min_blocks<S, MODE>())
 residual_kernel(const S* __restrict__ buf, Geom G, Coef<typename Real<S>::type> c,
-                P* __restrict__ snap, unsigned long long* __restrict__ slots, int nslots) {
+                P* __restrict__ snap, unsigned long long* __restrict__ slots,
+                double* __restrict__ out) {
     using R = typename Real<S>::type;
-    R dmax[4] = {0, 0, 0, 0}, amax[4] = {0, 0, 0, 0};
+    using B = typename Bits<R>::type;
+    B dmax[4] = {0, 0, 0, 0}, amax[4] = {0, 0, 0, 0};
     int bad = 0;
     const size_t n = (size_t)G.nx * G.ny;
     const int ntx = (G.nx + RES_THREADS - 1) / RES_THREADS;
@@ -1025,49 +1011,65 @@ residual_kernel(const S* __restrict__ buf, Geom G, Coef<typename Real<S>::type> 
             const R absv[4] = {M.ux, M.uy, c.T0 + M.Tp, c.C0 + M.Cp};
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                if (!finite_(phi[q])) bad = 1;
-                dmax[q] = max_(dmax[q], abs_(phi[q] - old[q]));
-                amax[q] = max_(amax[q], abs_(absv[q]));
+                if (bits_bad(ordered_bits(phi[q]))) bad = 1;
+                dmax[q] = max_bits(dmax[q], ordered_bits(phi[q] - old[q]));
+                amax[q] = max_bits(amax[q], ordered_bits(absv[q]));
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q) snap[q * n + k] = (P)phi[q];
         }
     }
-    // block maxima in R, one FP64 value per quantity for the slot
-    __shared__ R red[RES_THREADS / 32][9];
+    // block maxima, one FP64 value per quantity for the slot
+    __shared__ B red[RES_THREADS / 32][9];
+    __shared__ bool last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const R v[9] = {dmax[0], dmax[1], dmax[2], dmax[3], amax[0], amax[1], amax[2], amax[3], (R)bad};
+    const B v[9] = {dmax[0], dmax[1], dmax[2], dmax[3], amax[0], amax[1], amax[2], amax[3],
+                    bad ? ordered_bits(R(1)) : B(0)};
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-        const R r = warp_max(v[q]);
+        const B r = warp_max_bits(v[q]);
         if (lane == 0) red[warp][q] = r;
     }
     __syncthreads();
     if (threadIdx.x < 9) {
-        R s = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s = max_(s, red[w][threadIdx.x]);
-        const size_t b = ((size_t)blockIdx.y * gridDim.x + blockIdx.x) % (size_t)nslots;
-        atomicMax(slots + b * 9 + threadIdx.x, (unsigned long long)__double_as_longlong((double)s));
+        B s = 0;
+        for (int w = 0; w < RES_THREADS / 32; ++w) s = max_bits(s, red[w][threadIdx.x]);
+        const size_t b = ((size_t)blockIdx.y * gridDim.x + blockIdx.x) % (size_t)RES_SLOTS;
+        const unsigned long long d = (unsigned long long)__double_as_longlong(value_of(s));
+        if (d) atomicMax(slots + b * 9 + threadIdx.x, d);
+        __threadfence();                                 // the maxima before the count
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        last = atomicAdd(slots + RES_SLOTS * 9, 1ull) == (unsigned long long)gridDim.x * gridDim.y - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();                                     // the count before the maxima
+    // warp w folds the quantities w, w + 8: lane l the slots l, l + 32, ...
+    for (int q = warp; q < 9; q += RES_THREADS / 32) {
+        unsigned long long m = 0;
+        for (int b = lane; b < RES_SLOTS; b += 32)
+            m = max_bits(m, *(volatile unsigned long long*)(slots + (size_t)b * 9 + q));
+        m = warp_max_bits(m);
+        if (lane == 0) out[q] = __longlong_as_double((long long)m);
     }
 }
 
-// Clears the slots and launches pass 1 with the gather mode and the porous-field
+// Clears the slots and launches the pass with the gather mode and the porous-field
 // code fixed at compile time.
 template <typename S, typename P>
-cudaError_t launch_residual_pass1(const S* buf, const Geom& G, const Coef<typename Real<S>::type>& c,
-                                  int mode, P* snap, double* slots, int nslots, cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(slots, 0, (size_t)nslots * 9 * sizeof(double), st);
+cudaError_t launch_residual_pass(const S* buf, const Geom& G, const Coef<typename Real<S>::type>& c,
+                                 int mode, P* snap, double* slots, double* out, cudaStream_t st) {
+    cudaError_t e = cudaMemsetAsync(slots, 0, RES_SCRATCH * sizeof(double), st);
     if (e != cudaSuccess) return e;
     const dim3 grid = residual_grid(G);
     unsigned long long* sl = reinterpret_cast<unsigned long long*>(slots);
 #define LBM_RES_CASE(M)                                                                          \
     if (mode == M) {                                                                             \
         if (c.poro)                                                                              \
-            residual_kernel<S, true, P, M><<<grid, RES_THREADS, 0, st>>>(buf, G, c, snap, sl,     \
-                                                                        nslots);                 \
+            residual_kernel<S, true, P, M><<<grid, RES_THREADS, 0, st>>>(buf, G, c, snap, sl, out); \
         else                                                                                     \
-            residual_kernel<S, false, P, M><<<grid, RES_THREADS, 0, st>>>(buf, G, c, snap, sl,    \
-                                                                         nslots);                \
+            residual_kernel<S, false, P, M><<<grid, RES_THREADS, 0, st>>>(buf, G, c, snap, sl, out); \
         return cudaGetLastError();                                                               \
     }
     LBM_RES_CASE(GATHER_PULL_AB)
@@ -1077,9 +1079,5 @@ cudaError_t launch_residual_pass1(const S* buf, const Geom& G, const Coef<typena
 #undef LBM_RES_CASE
     return cudaErrorInvalidValue;
 }
-
-// Residual pass 2: one block folds partial[nblocks][9] into out[9].
-__global__ void __launch_bounds__(RES_THREADS)
-residual_final_kernel(const double* __restrict__ partial, int nblocks, double* __restrict__ out);
 
 }  // namespace lbm

@@ -43,7 +43,15 @@ struct WallSpec {
     int nee;                // 1: nodes on the walls (node stencil, trapezoidal mean)
 };
 
-constexpr int NUSH_THREADS = 512;
+constexpr int NUSH_THREADS = 64;      // line positions per block of the Nu / Sh pass
+constexpr int NUSH_MAX_BLOCKS = 256;  // blocks per wall at most
+// Doubles of d_out behind the results: the partial sums (Nu, Sh) of both walls' blocks,
+// and the count of finished blocks (zero between launches).
+constexpr int NUSH_SCRATCH = 4 * NUSH_MAX_BLOCKS + 1;
+inline unsigned nush_blocks(int positions) {
+    const int b = (positions + NUSH_THREADS - 1) / NUSH_THREADS;
+    return (unsigned)(b < NUSH_MAX_BLOCKS ? (b > 0 ? b : 1) : NUSH_MAX_BLOCKS);
+}
 constexpr int RES_THREADS = 256;
 
 struct LaunchCfg {
@@ -93,13 +101,13 @@ cudaError_t launch_fields(const void* buf, const Geom& G, const Coef<typename Re
                           int mode, int x0, int y0, int w, int h, double* out, cudaStream_t st);
 template <typename S>
 cudaError_t launch_nush(const void* buf, const Geom& G, const Coef<typename Real<S>::type>& c,
-                        int mode, const WallSpec& W, double* out, cudaStream_t st);
+                        int mode, const WallSpec& W, double* scratch, double* out, cudaStream_t st);
 // Nu / Sh on the bottom (Tw[0], Cw[0]) and top (Tw[1], Cw[1]) walls; out 4 doubles.
 template <typename S>
 cudaError_t launch_nush_tb(const void* buf, const Geom& G, const Coef<typename Real<S>::type>& c,
-                           int mode, const WallSpec& W, double* out, cudaStream_t st);
+                           int mode, const WallSpec& W, double* scratch, double* out, cudaStream_t st);
 // snap holds 4 * nx * ny values of the compute precision (FP64 for FP64 storage,
-// else FP32); partial must hold RES_SLOTS * 9 doubles; out 9 doubles.
+// else FP32); partial must hold RES_SCRATCH doubles; out 9 doubles.
 template <typename S>
 cudaError_t launch_residual(const void* buf, const Geom& G, const Coef<typename Real<S>::type>& c,
                             int mode, void* snap, double* partial, double* out,
@@ -109,7 +117,7 @@ cudaError_t launch_residual(const void* buf, const Geom& G, const Coef<typename 
 template <typename S>
 cudaError_t launch_halo(void* buf, const Geom& G, int row, int up, void* face, int pack,
                         cudaStream_t st);
-// Grid of the residual's first pass: 256-column tiles along x, one row per block
+// Grid of the residual pass: 256-column tiles along x, one row per block
 // along y (each block loops when ny exceeds the grid's y limit).
 inline dim3 residual_grid(const Geom& G) {
     const int ntx = (G.nx + RES_THREADS - 1) / RES_THREADS;
@@ -117,9 +125,10 @@ inline dim3 residual_grid(const Geom& G) {
     const int gy = rows < 65535 ? rows : 65535;
     return dim3((unsigned)ntx, (unsigned)(gy > 0 ? gy : 1), 1);
 }
-// Slots the first pass folds its block maxima into (atomically); the second pass
-// reduces the slots.
-constexpr int RES_SLOTS = 4096;
+// Slots the pass folds its block maxima into (atomically), and the doubles it needs:
+// the slots and the count of finished blocks.
+constexpr int RES_SLOTS = 64;
+constexpr int RES_SCRATCH = RES_SLOTS * 9 + 1;
 
 // Makes `dev` the calling thread's current device for the guard's lifetime and
 // restores the previous one afterwards (every entry point that touches a context's

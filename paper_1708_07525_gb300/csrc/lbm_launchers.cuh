@@ -233,15 +233,19 @@ cudaError_t launch_fields(const void* buf, const Geom& G, const Coef<typename Re
 
 template <typename S>
 cudaError_t launch_nush(const void* buf, const Geom& G, const Coef<typename Real<S>::type>& c,
-                        int mode, const WallSpec& W, double* out, cudaStream_t st) {
-    nush_kernel<S><<<1, NUSH_THREADS, 0, st>>>((const S*)buf, G, c, mode, W, out);
+                        int mode, const WallSpec& W, double* scratch, double* out, cudaStream_t st) {
+    const dim3 gr(nush_blocks(step_rows(G)), 2, 1);
+    nush_kernel<S, true><<<gr, NUSH_THREADS, 0, st>>>((const S*)buf, G, c, mode, W, scratch,
+                                                      (unsigned*)(scratch + NUSH_SCRATCH - 1), out);
     return cudaGetLastError();
 }
 
 template <typename S>
 cudaError_t launch_nush_tb(const void* buf, const Geom& G, const Coef<typename Real<S>::type>& c,
-                           int mode, const WallSpec& W, double* out, cudaStream_t st) {
-    nush_tb_kernel<S><<<1, NUSH_THREADS, 0, st>>>((const S*)buf, G, c, mode, W, out);
+                           int mode, const WallSpec& W, double* scratch, double* out, cudaStream_t st) {
+    const dim3 gr(nush_blocks(G.nx), 2, 1);
+    nush_kernel<S, false><<<gr, NUSH_THREADS, 0, st>>>((const S*)buf, G, c, mode, W, scratch,
+                                                       (unsigned*)(scratch + NUSH_SCRATCH - 1), out);
     return cudaGetLastError();
 }
 
@@ -250,11 +254,7 @@ cudaError_t launch_residual(const void* buf, const Geom& G, const Coef<typename 
                             int mode, void* snap, double* partial, double* out,
                             cudaStream_t st) {
     using R = typename Real<S>::type;
-    cudaError_t e = launch_residual_pass1<S, R>((const S*)buf, G, c, mode, (R*)snap, partial,
-                                                RES_SLOTS, st);
-    if (e != cudaSuccess) return e;
-    residual_final_kernel<<<1, RES_THREADS, 0, st>>>(partial, RES_SLOTS, out);
-    return cudaGetLastError();
+    return launch_residual_pass<S, R>((const S*)buf, G, c, mode, (R*)snap, partial, out, st);
 }
 
 template <typename S>
@@ -278,9 +278,10 @@ cudaError_t launch_halo(void* buf, const Geom& G, int row, int up, void* face, i
                                           const Coef<Real<S>::type>&, int, int, int, int, int, \
                                           double*, cudaStream_t);                              \
     template cudaError_t launch_nush<S>(const void*, const Geom&, const Coef<Real<S>::type>&,  \
-                                        int, const WallSpec&, double*, cudaStream_t);          \
+                                        int, const WallSpec&, double*, double*, cudaStream_t); \
     template cudaError_t launch_nush_tb<S>(const void*, const Geom&, const Coef<Real<S>::type>&,\
-                                           int, const WallSpec&, double*, cudaStream_t);       \
+                                           int, const WallSpec&, double*, double*,             \
+                                           cudaStream_t);                                      \
     template cudaError_t launch_residual<S>(const void*, const Geom&,                          \
                                             const Coef<Real<S>::type>&, int, void*, double*,   \
                                             double*, cudaStream_t);                            \

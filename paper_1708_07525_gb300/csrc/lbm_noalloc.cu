@@ -21,9 +21,10 @@ using namespace lbm;
 namespace {
 
 constexpr int NOALLOC_OUT = LBM_NOALLOC_MAX_BLOCKS * 9;   // offset of the 9 results
+static_assert(RES_SCRATCH <= NOALLOC_OUT, "the pass's slots fit before its results");
 
-// Partial maxima of up to LBM_NOALLOC_MAX_BLOCKS blocks (9 doubles each) plus the
-// 9 folded results.  Every GPU that loads the library holds this array (about
+// The slots of the residual pass's block maxima (RES_SCRATCH doubles of the room for
+// LBM_NOALLOC_MAX_BLOCKS times 9 that the header promises) plus the 9 folded results.  Every GPU that loads the library holds this array (about
 // 288 KiB) until the process exits.  In host code `noalloc_scratch` is only a
 // host-side stand-in for the symbol; its device address comes from
 // cudaGetSymbolAddress (see scratch_for_device).
@@ -57,12 +58,8 @@ template <typename S>
 cudaError_t launch(const CtxView& v, double* snap, double* scratch) {
     using R = typename Real<S>::type;
     const Coef<R>& c = coef_of(v, (R*)nullptr);
-    cudaError_t e = launch_residual_pass1<S, double>((const S*)v.buf, v.G, c, v.mode, snap, scratch,
-                                                     LBM_NOALLOC_MAX_BLOCKS, v.stream);
-    if (e != cudaSuccess) return e;
-    residual_final_kernel<<<1, RES_THREADS, 0, v.stream>>>(scratch, LBM_NOALLOC_MAX_BLOCKS,
-                                                          scratch + NOALLOC_OUT);
-    return cudaGetLastError();
+    return launch_residual_pass<S, double>((const S*)v.buf, v.G, c, v.mode, snap, scratch,
+                                           scratch + NOALLOC_OUT, v.stream);
 }
 
 lbm_status fail(lbm_ctx* ctx, lbm_status s, const char* m, const char* detail = "") {
@@ -88,8 +85,8 @@ lbm_status lbm_residual_noalloc(lbm_ctx* ctx, double* snapshot, int have_snapsho
     double* scratch = nullptr;
     cudaError_t e = scratch_for_device(v.device, &scratch);
     if (e != cudaSuccess) return fail(ctx, LBM_ERR_CUDA, "cudaGetSymbolAddress: ", cudaGetErrorString(e));
-    // The call clears the slots of the shared array before its first pass folds into
-    // them, and the fold writes all nine results.
+    // The call clears the slots of the shared array before its pass folds into them, and
+    // the pass's last block writes all nine results.
     switch (v.prec) {
         case LBM_F64: e = launch<double>(v, snapshot, scratch); break;
         case LBM_F32: e = launch<float>(v, snapshot, scratch); break;
