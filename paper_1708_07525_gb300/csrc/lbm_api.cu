@@ -62,22 +62,32 @@ Coef<R> make_coef(const lbm_params& P) {
     c.l0 = (R)l0;
     c.l0sq = (R)(l0 * l0);
     c.l1 = (R)l1;
-    c.drag_lin = (R)(eps * P.nu / P.K);                     // Eq. 5
-    c.drag_quad = (R)(eps * P.Feps / std::sqrt(P.K));
-    c.s1 = (R)P.s[1]; c.s2 = (R)P.s[2]; c.s3 = (R)P.s[3]; c.s4 = (R)P.s[4];
-    c.s5 = (R)P.s[5]; c.s6 = (R)P.s[6]; c.s7 = (R)P.s[7]; c.s8 = (R)P.s[8];
-    c.za1 = (R)P.zeta[1]; c.za2 = (R)P.zeta[2]; c.za3 = (R)P.zeta[3]; c.za4 = (R)P.zeta[4];
-    c.ed1 = (R)P.eta[1]; c.ed2 = (R)P.eta[2]; c.ed3 = (R)P.eta[3]; c.ed4 = (R)P.eta[4];
-    // 1 - s/2 factors of the forcing / source terms (Eqs. 10, 21, 22), in the compute precision
-    c.h1 = (R)(1.0 - 0.5 * P.s[1]); c.h2 = (R)(1.0 - 0.5 * P.s[2]);
-    c.h3 = (R)(1.0 - 0.5 * P.s[3]); c.h4 = (R)(1.0 - 0.5 * P.s[4]);
-    c.h5 = (R)(1.0 - 0.5 * P.s[5]); c.h6 = (R)(1.0 - 0.5 * P.s[6]);
-    c.h7 = (R)(1.0 - 0.5 * P.s[7]); c.h8 = (R)(1.0 - 0.5 * P.s[8]);
-    c.hz1 = (R)(1.0 - 0.5 * P.zeta[1]); c.hz2 = (R)(1.0 - 0.5 * P.zeta[2]);
-    c.he1 = (R)(1.0 - 0.5 * P.eta[1]); c.he2 = (R)(1.0 - 0.5 * P.eta[2]);
+    c.ndrag_lin = (R)(-eps * P.nu / P.K);                   // Eq. 5
+    c.ndrag_quad = (R)(-eps * P.Feps / std::sqrt(P.K));
+    c.half_epsGx = (R)(0.5 * eps * P.Gx);
+    c.epsGx = (R)(eps * P.Gx);
+    // relaxation rates s and forcing factors 1 - s / 2 (Eqs. 10, 21, 22) with the factors of
+    // M^-1 and N^-1, in the compute precision (collide_flow, collide_d2q5)
+    auto h = [](double s) { return 1.0 - 0.5 * s; };
+    c.k1 = (R)(P.s[1] / 36.0);  c.k1F = (R)(-h(P.s[1]) / 6.0);
+    c.k2 = (R)(P.s[2] / 12.0);  c.k2F = (R)(h(P.s[2]) / 6.0);
+    c.k4 = (R)(P.s[4] / 12.0);  c.k4F = (R)(h(P.s[4]) / 12.0);
+    c.k6 = (R)(P.s[6] / 12.0);  c.k6F = (R)(h(P.s[6]) / 12.0);
+    c.k7 = (R)(P.s[7] / 4.0);   c.k7F = (R)(-h(P.s[7]) / 2.0);
+    c.k8 = (R)(P.s[8] / 4.0);   c.k8F = (R)(-h(P.s[8]) / 4.0);
+    auto scalar = [&](const double r[5]) {
+        CoefScalar<R> k;
+        k.b1 = (R)(r[1] / 2.0);  k.q1 = (R)(-h(r[1]) / 2.0);
+        k.b2 = (R)(r[2] / 2.0);  k.q2 = (R)(-h(r[2]) / 2.0);
+        k.b3 = (R)(r[3] / 20.0);
+        k.b4 = (R)(r[4] / 4.0);
+        return k;
+    };
+    c.zs = scalar(P.zeta);
+    c.es = scalar(P.eta);
     // Eqs. 24 / 25 (model A: Eqs. 30 / 31): n_eq,3 = c3 Phi
-    c.c3T = (R)(P.model_a ? (5.0 * P.varpi - 4.0) * P.sigma : 5.0 * P.varpi - 4.0 * P.sigma);
-    c.c3C = (R)(P.model_a ? (5.0 * P.varpi - 4.0) * eps : 5.0 * P.varpi - 4.0 * eps);
+    c.nc3T = (R)(P.model_a ? (4.0 - 5.0 * P.varpi) * P.sigma : 4.0 * P.sigma - 5.0 * P.varpi);
+    c.nc3C = (R)(P.model_a ? (4.0 - 5.0 * P.varpi) * eps : 4.0 * eps - 5.0 * P.varpi);
     const double w = 0.25 * P.varpi;                        // w~_1..4 (Sec. 3.2)
     // anti-bounce-back constant g_q^eq + g_opp^eq at the wall value: 2 w~ Phi_w (Eq. 28),
     // 2 w~ sigma T_w / 2 w~ eps C_w for model A; in deviations from Phi0
@@ -119,7 +129,6 @@ Coef<R> make_coef(const lbm_params& P) {
 }
 template Coef<float> make_coef<float>(const lbm_params&);
 template Coef<double> make_coef<double>(const lbm_params&);
-template Coef<f2> make_coef<f2>(const lbm_params&);
 }  // namespace lbm
 
 namespace {
@@ -186,7 +195,6 @@ struct lbm_ctx {
     bool slab = false;              // a slab of a cavity split along y (lbm_create_slab)
     Coef<double> cd{};
     Coef<float> cf{};
-    Coef<f2> cp{};                  // 16-bit storage: cf as pairs (two nodes per thread)
     LaunchCfg L{};
     int graph_chunk = 0;
     bool round_nearest = false;     // 16-bit storage: nearest-even instead of stochastic
@@ -626,8 +634,6 @@ lbm_status create_core(const lbm_params* params, const lbm_options* opt, int sla
     c->cf = make_coef<float>(c->P);
     c->round_nearest = O.round_nearest != 0;
     c->cf.sr = c->round_nearest ? 0 : 1;
-    c->cp = make_coef<f2>(c->P);
-    c->cp.sr = c->cf.sr;
     // rounding streams keyed by the node's index in the undivided cavity
     c->cf.seed_off = (long long)(c->slab_y0 - c->G.jb) * c->G.pitch;
     int bx = O.block_x, by = O.block_y;
@@ -646,7 +652,7 @@ lbm_status create_core(const lbm_params* params, const lbm_options* opt, int sla
     c->L.aux = nullptr;
     // 16-bit storage takes the two-nodes-per-thread kernels, except on slabs, whose rows
     // all run the one-node kernel (the same arithmetic as a one-node whole cavity)
-    c->L.pair = (c->prec == LBM_BF16 || c->prec == LBM_F16) && !slab ? &c->cp : nullptr;
+    c->L.pair = (c->prec == LBM_BF16 || c->prec == LBM_F16) && !slab;
     // a second stream lets the small ring launch of a split step run beside the inner one;
     // without it both go to the context's stream
     if (cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking) == cudaSuccess &&
@@ -1206,8 +1212,6 @@ lbm_status lbm_load(lbm_ctx* c, const void* buf, size_t len) {
     c->cd = make_coef<double>(c->P);
     c->cf = make_coef<float>(c->P);
     c->cf.sr = c->round_nearest ? 0 : 1;
-    c->cp = make_coef<f2>(c->P);
-    c->cp.sr = c->cf.sr;
     c->cf.seed_off = (long long)(c->slab_y0 - c->G.jb) * c->G.pitch;
     c->cd.poro = (c->poro && c->rsz == 8) ? (const double*)c->poro : nullptr;
     c->cf.poro = (c->poro && c->rsz == 4) ? (const float*)c->poro : nullptr;

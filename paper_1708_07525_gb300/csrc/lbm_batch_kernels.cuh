@@ -210,8 +210,8 @@ batch_residual_kernel(const BatchInst<typename Real<S>::type>* __restrict__ tabl
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     if (!finite_(phi[q])) bad = 1;
-                    dmax[q] = max_(dmax[q], abs_(phi[q] - old[q]));
-                    amax[q] = max_(amax[q], abs_(absv[q]));
+                    dmax[q] = fmaxf(dmax[q], fabsf(phi[q] - old[q]));
+                    amax[q] = fmaxf(amax[q], fabsf(absv[q]));
                 }
 #pragma unroll
                 for (int q = 0; q < 4; ++q) I.snap[q * n + kk] = phi[q];
@@ -228,7 +228,7 @@ batch_residual_kernel(const BatchInst<typename Real<S>::type>* __restrict__ tabl
         __syncthreads();
         if (threadIdx.x < 9) {
             R s = 0;
-            for (int w = 0; w < BATCH_THREADS / 32; ++w) s = max_(s, red[w][threadIdx.x]);
+            for (int w = 0; w < BATCH_THREADS / 32; ++w) s = fmaxf(s, red[w][threadIdx.x]);
             partial[(size_t)tile * 9 + threadIdx.x] = (double)s;
         }
     }
@@ -241,22 +241,23 @@ batch_residual_fold_kernel(const BatchInst<R>* __restrict__ table, const int* __
                            const double* __restrict__ partial, double* __restrict__ out) {
     const int k = blockIdx.x;
     const int b0 = table[k].tile_begin, nt = ntiles[k];
-    __shared__ double red[BATCH_THREADS / 32][9];
-    double v[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+    __shared__ unsigned long long red[BATCH_THREADS / 32][9];
+    // non-negative values by their bit patterns (integer maxima, off the FP64 pipe)
+    unsigned long long v[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     for (int t = threadIdx.x; t < nt; t += blockDim.x)
 #pragma unroll
-        for (int q = 0; q < 9; ++q) v[q] = fmax(v[q], partial[(size_t)(b0 + t) * 9 + q]);
+        for (int q = 0; q < 9; ++q) v[q] = max_bits(v[q], ordered_bits(partial[(size_t)(b0 + t) * 9 + q]));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-        const double r = warp_max(v[q]);
+        const unsigned long long r = warp_max_bits(v[q]);
         if (lane == 0) red[warp][q] = r;
     }
     __syncthreads();
     if (threadIdx.x < 9) {
-        double s = 0;
-        for (int w = 0; w < BATCH_THREADS / 32; ++w) s = fmax(s, red[w][threadIdx.x]);
-        out[(size_t)k * 9 + threadIdx.x] = s;
+        unsigned long long s = 0;
+        for (int w = 0; w < BATCH_THREADS / 32; ++w) s = max_bits(s, red[w][threadIdx.x]);
+        out[(size_t)k * 9 + threadIdx.x] = value_of(s);
     }
 }
 
@@ -288,10 +289,8 @@ batch_nush_kernel(const BatchInst<typename Real<S>::type>* __restrict__ table,
                 }
                 R f[9], g[5], h[5];
                 gather<false>(mode, buf, G, far ? G.nx - 1 - q : q, j, I.c, f, g, h);
-                const R sg = ((g[0] + g[1]) + (g[2] + g[3])) + g[4];
-                const R sh = ((h[0] + h[1]) + (h[2] + h[3])) + h[4];
-                T[q] = W.T0 + (double)(sg * I.c.inv_sigma);
-                C[q] = W.C0 + (double)(sh * I.c.inv_eps);
+                T[q] = W.T0 + (double)mul_(sum5(g), I.c.inv_sigma);
+                C[q] = W.C0 + (double)mul_(sum5(h), I.c.inv_eps);
             }
             if (W.nee) {
                 const double w = (j == 0 || j == G.ny - 1) ? 0.5 : 1.0;

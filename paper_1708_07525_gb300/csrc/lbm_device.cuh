@@ -54,14 +54,6 @@ __device__ __forceinline__ uint32_t mix32(uint32_t x) {
 template <typename R> __device__ __forceinline__ R sqrt_(R x);
 template <> __device__ __forceinline__ float sqrt_(float x) { return sqrtf(x); }
 template <> __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
-// |x|, max(a, b) and finiteness in the precision of the argument (FP32 stays on the
-// FP32 pipes; GB300's FP64 pipe is narrow).
-template <typename R> __device__ __forceinline__ R abs_(R x);
-template <> __device__ __forceinline__ float abs_(float x) { return fabsf(x); }
-template <> __device__ __forceinline__ double abs_(double x) { return fabs(x); }
-template <typename R> __device__ __forceinline__ R max_(R a, R b);
-template <> __device__ __forceinline__ float max_(float a, float b) { return fmaxf(a, b); }
-template <> __device__ __forceinline__ double max_(double a, double b) { return fmax(a, b); }
 template <typename R> __device__ __forceinline__ bool finite_(R x);
 template <> __device__ __forceinline__ bool finite_(float x) { return fabsf(x) <= 3.402823466e38f; }
 template <> __device__ __forceinline__ bool finite_(double x) { return fabs(x) <= 1.7976931348623157e308; }
@@ -161,13 +153,27 @@ __device__ __forceinline__ uint32_t node_seed(size_t node, R a, R b) {
     return mix32(ia ^ mix32(ib ^ mix32((uint32_t)node ^ (uint32_t)(node >> 32) * 0x27D4EB2Fu)));
 }
 
-// ---- two nodes per thread ----------------------------------------------------------
-// f2: the FP32 values of one quantity at two x-adjacent nodes, computed with the packed
-// FP32x2 instructions of sm_100 and later (one add, multiply or fused multiply-add for
-// both nodes).  Products are kept unevaluated (f2m) until they meet an addition or a
-// subtraction, which then becomes one fused multiply-add, as a compiler contracts
-// a * b + c in scalar code.  Division and square root act per component.  The scalar
-// collision and macroscopic code (collide, macro) is instantiated with R = f2.
+// ---- arithmetic with every rounding written out ------------------------------------------
+// One node's step is written with these operations only, so that its result does not hang
+// on which products and sums a compiler fuses: the one-node kernels, the kernels with two
+// nodes per thread and the batch kernels give the same bits, whatever surrounds the
+// arithmetic.  fma_(a, b, c) = a b + c and fnma_(a, b, c) = c - a b round once.
+__device__ __forceinline__ float add_(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub_(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float fnma_(float a, float b, float c) { return __fmaf_rn(-a, b, c); }
+__device__ __forceinline__ double add_(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub_(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double fnma_(double a, double b, double c) { return __fma_rn(-a, b, c); }
+
+// f2: the FP32 values of one quantity at two nodes, computed with the packed FP32x2
+// instructions of sm_100 and later (one add, multiply or fused multiply-add for both
+// nodes; each component rounds as the scalar operation does).  Constants stay scalar and
+// are written R(c): an instruction takes one value for both components as it takes an
+// immediate, where a pair of constants has to be brought into registers first.
 struct f2 {
     float2 v;
     f2() = default;
@@ -176,44 +182,72 @@ struct f2 {
     __host__ __device__ explicit f2(T s) : v(make_float2((float)s, (float)s)) {}
 };
 #ifdef __CUDACC__
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
-struct f2m {
-    float2 a, b;
-    __device__ __forceinline__ operator f2() const { return f2(__fmul2_rn(a, b)); }
-};
-__device__ __forceinline__ f2m operator*(f2 a, f2 b) { return f2m{a.v, b.v}; }
-__device__ __forceinline__ f2m operator*(f2m a, f2 b) { return f2m{f2(a).v, b.v}; }
-__device__ __forceinline__ f2m operator*(f2 a, f2m b) { return f2m{a.v, f2(b).v}; }
-__device__ __forceinline__ f2m operator*(f2m a, f2m b) { return f2m{f2(a).v, f2(b).v}; }
-__device__ __forceinline__ f2 operator+(f2 a, f2 b) { return f2(__fadd2_rn(a.v, b.v)); }
-__device__ __forceinline__ f2 operator-(f2 a, f2 b) {
+__device__ __forceinline__ f2 add_(f2 a, f2 b) { return f2(__fadd2_rn(a.v, b.v)); }
+__device__ __forceinline__ f2 sub_(f2 a, f2 b) {
     return f2(__ffma2_rn(b.v, make_float2(-1.0f, -1.0f), a.v));   // round(a - b) exactly
 }
-__device__ __forceinline__ f2 operator+(f2m p, f2 c) { return f2(__ffma2_rn(p.a, p.b, c.v)); }
-__device__ __forceinline__ f2 operator+(f2 c, f2m p) { return f2(__ffma2_rn(p.a, p.b, c.v)); }
-__device__ __forceinline__ f2 operator-(f2 c, f2m p) { return f2(__ffma2_rn(neg2(p.a), p.b, c.v)); }
-__device__ __forceinline__ f2 operator-(f2m p, f2 c) { return f2(__ffma2_rn(p.a, p.b, neg2(c.v))); }
-__device__ __forceinline__ f2 operator+(f2m p, f2m q) { return f2(__ffma2_rn(p.a, p.b, f2(q).v)); }
-__device__ __forceinline__ f2 operator-(f2m p, f2m q) {
-    return f2(__ffma2_rn(neg2(q.a), q.b, f2(p).v));
-}
-__device__ __forceinline__ f2 operator-(f2 a) { return f2(neg2(a.v)); }
-__device__ __forceinline__ f2 operator-(f2m p) { return f2m{neg2(p.a), p.b}; }
-__device__ __forceinline__ f2& operator+=(f2& a, f2 b) { return a = a + b; }
-__device__ __forceinline__ f2& operator-=(f2& a, f2 b) { return a = a - b; }
-__device__ __forceinline__ f2& operator+=(f2& a, f2m b) { return a = a + b; }
-__device__ __forceinline__ f2& operator-=(f2& a, f2m b) { return a = a - b; }
-__device__ __forceinline__ f2 operator/(f2 a, f2 b) { return f2(make_float2(a.v.x / b.v.x, a.v.y / b.v.y)); }
-template <> __device__ __forceinline__ f2 sqrt_(f2 x) {
-    return f2(make_float2(sqrtf(x.v.x), sqrtf(x.v.y)));
+__device__ __forceinline__ f2 mul_(f2 a, f2 b) { return f2(__fmul2_rn(a.v, b.v)); }
+__device__ __forceinline__ f2 fma_(f2 a, f2 b, f2 c) { return f2(__ffma2_rn(a.v, b.v, c.v)); }
+__device__ __forceinline__ f2 fnma_(f2 a, f2 b, f2 c) {
+    return f2(__ffma2_rn(make_float2(-a.v.x, -a.v.y), b.v, c.v));
 }
 #endif
+
+// sqrt(x) and 1 / x of a normal x > 0, rounded to nearest.
+//   FP32: CUDA's root and division in the one-node kernels, which have all loads issued by
+//   the time these functions' branches come up (within one basic block the compiler
+//   put loads between the sums that they feed: a 256^2 step took 4.5 instead of 3.4 us).
+//   f2: per component, or (FLAT) without a branch for both at once by Markstein's sequences
+//   (P. Markstein, "IA-64 and Elementary Functions", 2000) from the special-function unit's
+//   approximation y: Newton steps on g ~ sqrt(x) and h ~ 1 / (2 sqrt(x)), or on y ~ 1 / x, and
+//   a last correction from the exact residual, which rounds as the exact result does.
+//   FP64: the binomial series of (1 - e)^(-1/2) and (1 - e)^(-1) to second order in the
+//   error e of the approximation (below 2^-19): within an ulp, in 5 and 3 operations.
+__device__ __forceinline__ float rsqrt_seed(float x) { float y; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+__device__ __forceinline__ float rcp_seed(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+__device__ __forceinline__ double rsqrt_seed(double x) { double y; asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x)); return y; }
+__device__ __forceinline__ double rcp_seed(double x) { double y; asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x)); return y; }
+
+template <bool FLAT> __device__ __forceinline__ float sqrt_pos(float x) { return sqrtf(x); }
+template <bool FLAT> __device__ __forceinline__ float rcp_pos(float x) { return 1.0f / x; }
+template <bool FLAT> __device__ __forceinline__ double sqrt_pos(double x) {
+    const double y = rsqrt_seed(x), g = mul_(x, y), e = fnma_(g, y, 1.0);
+    return fma_(mul_(g, e), fma_(e, 0.375, 0.5), g);
+}
+template <bool FLAT> __device__ __forceinline__ double rcp_pos(double x) {
+    const double y = rcp_seed(x), e = fnma_(x, y, 1.0);
+    return fma_(y, fma_(e, e, e), y);
+}
+#ifdef __CUDACC__
+template <bool FLAT> __device__ __forceinline__ f2 sqrt_pos(f2 x) {
+    if (!FLAT) return f2(make_float2(sqrtf(x.v.x), sqrtf(x.v.y)));
+    const f2 y = f2(make_float2(rsqrt_seed(x.v.x), rsqrt_seed(x.v.y)));
+    const f2 g = mul_(x, y), h = mul_(y, f2(0.5f)), r = fnma_(g, h, f2(0.5f));
+    const f2 g1 = fma_(g, r, g), h1 = fma_(h, r, h);
+    return fma_(fnma_(g1, g1, x), h1, g1);
+}
+template <bool FLAT> __device__ __forceinline__ f2 rcp_pos(f2 x) {
+    if (!FLAT) return f2(make_float2(1.0f / x.v.x, 1.0f / x.v.y));
+    const f2 y = f2(make_float2(rcp_seed(x.v.x), rcp_seed(x.v.y)));
+    const f2 y1 = fma_(y, fnma_(x, y, f2(1.0f)), y);
+    return fma_(y1, fnma_(x, y1, f2(1.0f)), y1);
+}
+#endif
+// Added to |v|^2 under the root, which is then never zero, and whose residual in Markstein's
+// sequence is never subnormal: far below half a unit of what the root is added to (Eq. 18's
+// l0^2 >= 1/4 after a factor l1, Eq. 5's drag).
+template <typename R> __device__ __forceinline__ R tiny_() { return R(1e-28); }
+template <> __device__ __forceinline__ double tiny_<double>() { return 1e-300; }
 
 // Compute type for a storage type: FP64 stays FP64, everything else is FP32.
 template <typename S> struct Real { using type = float; };
 template <> struct Real<double> { using type = double; };
 
 // ---- per-instance constants (prepared on the host, passed by value) ------------
+template <typename R>
+struct CoefScalar {
+    R b1, q1, b2, q2, b3, b4;
+};
 template <typename R>
 struct Coef {
     R T0, C0;
@@ -222,13 +256,17 @@ struct Coef {
     R inv_eps_f;               // 1/eps for the flow equilibria (Eqs. 14, 15)
     R gbT, gbC, Gx;            // Eq. 6 (+ optional constant Gx)
     R l0, l0sq, l1;            // Eq. 19
-    R drag_lin, drag_quad;     // eps nu / K and eps F_eps / sqrt(K) (Eq. 5)
-    R s1, s2, s3, s4, s5, s6, s7, s8;   // Lambda (s_rho plays no role: m_0 is conserved)
-    R h1, h2, h3, h4, h5, h6, h7, h8;   // 1 - s_k / 2, the factors of the forcing (Eq. 10)
-    R za1, za2, za3, za4;      // Theta (zeta_0 plays no role)
-    R ed1, ed2, ed3, ed4;      // Q
-    R hz1, hz2, he1, he2;      // 1 - zeta_k / 2, 1 - eta_k / 2 (source terms of Eqs. 21-22)
-    R c3T, c3C;                // 5 varpi - 4 sigma, 5 varpi - 4 eps (Eqs. 24, 25)
+    R ndrag_lin, ndrag_quad;   // -eps nu / K and -eps F_eps / sqrt(K) (Eq. 5)
+    R half_epsGx, epsGx;       // eps Gx / 2, eps Gx
+    // Relaxation and forcing of the moments with the factors of M^-1 (Eq. 10): Lambda_k
+    // and 1 - Lambda_k / 2 times 1/36 (e, and 3/36 for eps), 1/12 (q), 1/4 (nu), see
+    // collide_flow().  s_rho and s_j play no role: rho is conserved, and the momentum gains
+    // exactly F whatever s_j (Eq. 17).
+    R k1, k1F, k2, k2F, k4, k4F, k6, k6F, k7, k7F, k8, k8F;
+    // Theta, Q and the source factors with those of N^-1 (Eqs. 21, 22, 27): r_1 / 2,
+    // -(1 - r_1 / 2) / 2, the same for r_2, r_3 / 20, r_4 / 4.
+    CoefScalar<R> zs, es;
+    R nc3T, nc3C;              // 4 sigma - 5 varpi, 4 eps - 5 varpi (Eqs. 24, 25)
     // Per wall side (0 left, 1 right, 2 bottom, 3 top): 2 w~ (Phi_w - Phi0) with
     // w~ = varpi / 4, the anti-bounce-back constant in deviations.
     R wallT[4], wallC[4];
@@ -269,14 +307,16 @@ __device__ __forceinline__ void porous_at(Coef<R>& c, size_t self, size_t plane)
     c.half_eps = R(0.5) * e;
     c.inv_eps = R(1) / e;
     c.inv_eps_f = c.inv_eps;
-    c.drag_lin = e * c.nu / K;
-    c.drag_quad = e * Fe / sqrt_(K);
-    c.l0 = R(0.5) * (R(1) + R(0.5) * c.drag_lin);
+    c.ndrag_lin = -(e * c.nu / K);
+    c.ndrag_quad = -(e * Fe / sqrt_(K));
+    c.half_epsGx = c.half_eps * c.Gx;
+    c.epsGx = e * c.Gx;
+    c.l0 = R(0.5) * (R(1) - R(0.5) * c.ndrag_lin);
     c.l0sq = c.l0 * c.l0;
-    c.l1 = R(0.5) * c.drag_quad;
-    c.c3C = c.varpi5 - R(4) * e;
-    c.aC0 = (e - c.c3C) * R(0.2);
-    c.aC1 = e * R(0.2) + c.c3C * R(0.05);
+    c.l1 = R(-0.5) * c.ndrag_quad;
+    c.nc3C = R(4) * e - c.varpi5;
+    c.aC0 = (e + c.nc3C) * R(0.2);
+    c.aC1 = e * R(0.2) - c.nc3C * R(0.05);
 }
 
 // Macroscopic quantities of one node from pre-collision deviations.
@@ -285,31 +325,34 @@ struct Macro {
     R rho, ux, uy, Tp, Cp, Fx, Fy;   // rho' (deviation), u, T - T0, C - C0, F
 };
 
+// Sums and differences of opposite populations of one lattice; collide_flow() and
+// collide_d2q5() need the ones that macro() forms again (the compiler shares them).
 template <typename R>
-__device__ __forceinline__ Macro<R> macro(const Coef<R>& c, const R f[9], const R g[5],
+__device__ __forceinline__ R sum5(const R d[5]) {
+    return add_(d[0], add_(add_(d[1], d[3]), add_(d[2], d[4])));
+}
+
+template <bool FLAT = false, typename K, typename R>
+__device__ __forceinline__ Macro<R> macro(const Coef<K>& c, const R f[9], const R g[5],
                                           const R h[5]) {
     Macro<R> o;
-    R rho = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];  // Eq. 16
-    R jx = (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]);
-    R jy = (f[2] - f[4]) + (f[5] + f[6]) - (f[7] + f[8]);
-    R Tp = (((g[0] + g[1]) + (g[2] + g[3])) + g[4]) * c.inv_sigma;   // Eq. 26
-    R Cp = (((h[0] + h[1]) + (h[2] + h[3])) + h[4]) * c.inv_eps;
-    R Gy = c.gbT * Tp + c.gbC * Cp;                                  // Eq. 6
-    R vx = jx + c.half_eps * c.Gx;                                   // Eq. 19, rho0 = 1
-    R vy = jy + c.half_eps * Gy;
-    R vm = sqrt_(vx * vx + vy * vy);
-    R den = c.l0 + sqrt_(c.l0sq + c.l1 * vm);                       // Eq. 18
-    const R inv_den = R(1) / den;
-    R ux = vx * inv_den, uy = vy * inv_den;
-    R um = sqrt_(ux * ux + uy * uy);
-    R drag = c.drag_lin + c.drag_quad * um;                          // Eq. 5
-    o.rho = rho;
-    o.ux = ux;
-    o.uy = uy;
-    o.Tp = Tp;
-    o.Cp = Cp;
-    o.Fx = c.eps * c.Gx - drag * ux;
-    o.Fy = c.eps * Gy - drag * uy;
+    const R p = add_(add_(f[1], f[3]), add_(f[2], f[4])), d = add_(add_(f[5], f[7]), add_(f[6], f[8]));
+    const R D57 = sub_(f[5], f[7]), D68 = sub_(f[6], f[8]);
+    const R jx = add_(add_(sub_(f[1], f[3]), D57), sub_(f[8], f[6]));
+    const R jy = add_(sub_(f[2], f[4]), add_(D57, D68));
+    o.rho = add_(f[0], add_(p, d));                                  // Eq. 16
+    o.Tp = mul_(sum5(g), R(c.inv_sigma));                               // Eq. 26
+    o.Cp = mul_(sum5(h), R(c.inv_eps));
+    const R Gy = fma_(R(c.gbT), o.Tp, mul_(R(c.gbC), o.Cp));               // Eq. 6
+    const R vx = add_(jx, R(c.half_epsGx));                             // Eq. 19, rho0 = 1
+    const R vy = fma_(R(c.half_eps), Gy, jy);
+    const R vm = sqrt_pos<FLAT>(fma_(vx, vx, fma_(vy, vy, tiny_<R>())));
+    const R inv_den = rcp_pos<FLAT>(add_(R(c.l0), sqrt_pos<FLAT>(fma_(R(c.l1), vm, R(c.l0sq)))));   // Eq. 18
+    o.ux = mul_(vx, inv_den);
+    o.uy = mul_(vy, inv_den);
+    const R ndrag = fma_(R(c.ndrag_quad), mul_(vm, inv_den), R(c.ndrag_lin));        // Eq. 5, |u| = |v| / den
+    o.Fx = fma_(ndrag, o.ux, R(c.epsGx));
+    o.Fy = fma_(ndrag, o.uy, mul_(R(c.eps), Gy));
     return o;
 }
 
@@ -317,107 +360,90 @@ __device__ __forceinline__ Macro<R> macro(const Coef<R>& c, const R f[9], const 
 // (0, X_x, X_y, 0, 0) of Eq. 27), written as d* = d - N^-1 [Theta (n - n_eq)
 // - (I - Theta/2) S] so that only the change is rounded; the zeroth moment
 // (cap * Phi) is conserved exactly, its change is set to zero.  N^-1 uses the
-// orthogonality of N: N^-1 = N^T D^-1, D = diag(5, 2, 2, 20, 4).
-// Pp = Phi - Phi0, P = Phi (Phi = T or C), c3 = 5 varpi - 4 cap.
-template <typename R>
-__device__ __forceinline__ void collide_d2q5(R d[5], R Pp, R P, R ux, R uy, R Xx, R Xy,
-                                             R r1, R r2, R r3, R r4, R c3, R q1, R q2) {
-    const R n1 = d[1] - d[3];
-    const R n2 = d[2] - d[4];
-    const R n3 = ((d[1] + d[2]) + (d[3] + d[4])) - R(4) * d[0];
-    const R n4 = (d[1] - d[2]) + (d[3] - d[4]);
-    const R k1 = r1 * (n1 - ux * P) - q1 * Xx;   // q_k = 1 - r_k / 2
-    const R k2 = r2 * (n2 - uy * P) - q2 * Xy;
-    const R k3 = r3 * (n3 - c3 * Pp);
-    const R k4 = r4 * n4;
-    const R b1 = k1 * R(0.5), b2 = k2 * R(0.5), b3 = k3 * R(0.05), b4 = k4 * R(0.25);
-    d[0] += R(4) * b3;
-    d[1] -= b1 + b3 + b4;
-    d[2] -= b2 + b3 - b4;
-    d[3] -= -b1 + b3 + b4;
-    d[4] -= -b2 + b3 - b4;
+// orthogonality of N: N^-1 = N^T D^-1, D = diag(5, 2, 2, 20, 4), whose factors r carries.
+// Pp = Phi - Phi0, nc3 = 4 cap - 5 varpi, (Px, Py) = Phi u, (Xx, Xy) its change.
+template <typename K, typename R>
+__device__ __forceinline__ void collide_d2q5(R d[5], R Pp, R Px, R Py, R Xx, R Xy,
+                                             const CoefScalar<K>& r, K nc3) {
+    const R p13 = add_(d[1], d[3]), p24 = add_(d[2], d[4]);
+    const R n3 = fma_(R(-4), d[0], add_(p13, p24));
+    const R n4 = sub_(p13, p24);
+    const R b1 = fma_(R(r.b1), sub_(sub_(d[1], d[3]), Px), mul_(R(r.q1), Xx));
+    const R b2 = fma_(R(r.b2), sub_(sub_(d[2], d[4]), Py), mul_(R(r.q2), Xy));
+    const R b3 = mul_(R(r.b3), fma_(R(nc3), Pp, n3));
+    const R b4 = mul_(R(r.b4), n4);
+    const R X = add_(b3, b4), Y = sub_(b3, b4);
+    d[0] = fma_(R(4), b3, d[0]);
+    d[1] = sub_(d[1], add_(X, b1));
+    d[2] = sub_(d[2], add_(Y, b2));
+    d[3] = sub_(d[3], sub_(X, b1));
+    d[4] = sub_(d[4], sub_(Y, b2));
 }
 
 // The collision of one node, in place on the deviations f, g, h: collide_flow (the D2Q9
 // part), then collide_scalars; collide() does both.  hist = (T u_x, T u_y, C u_x, C u_y)
 // at the previous step; updated.  The D2Q9 part is Eq. 10 written as
 // f* = f - M^-1 [Lambda (m - m_eq) - (I - Lambda/2) S] (only the change is rounded; the
-// density moment is conserved exactly).
-template <typename R>
-__device__ __forceinline__ void collide_flow(const Coef<R>& c, const Macro<R>& M, R f[9]) {
-    const R ux = M.ux, uy = M.uy, Fx = M.Fx, Fy = M.Fy, rho = M.rho;
-    const R ie = c.inv_eps_f;
-    // m = M f (Eq. 13), deviation part; m_0 = rho' is not needed
-    const R fa = (f[1] + f[2]) + (f[3] + f[4]);
-    const R fd = (f[5] + f[6]) + (f[7] + f[8]);
-    const R m1 = R(2) * fd - fa - R(4) * f[0];
-    const R m2 = R(4) * f[0] - R(2) * fa + fd;
-    const R m3 = (f[1] - f[3]) + (f[5] - f[6]) + (f[8] - f[7]);
-    const R m4 = R(2) * (f[3] - f[1]) + (f[5] - f[6]) + (f[8] - f[7]);
-    const R m5 = (f[2] - f[4]) + (f[5] + f[6]) - (f[7] + f[8]);
-    const R m6 = R(2) * (f[4] - f[2]) + (f[5] + f[6]) - (f[7] + f[8]);
-    const R m7 = (f[1] - f[2]) + (f[3] - f[4]);
-    const R m8 = (f[5] - f[6]) + (f[7] - f[8]);
-    // m_eq (Eq. 14, alpha1 = 1, alpha2 = -3, rho0 = 1) minus its rest part, and S (Eq. 15)
-    const R u2e = (ux * ux + uy * uy) * ie;
-    const R uF = (ux * Fx + uy * Fy) * ie;
-    const R e1 = R(-2) * rho + R(3) * u2e;
-    const R e2 = rho - R(3) * u2e;
-    const R e7 = (ux * ux - uy * uy) * ie;
-    const R e8 = ux * uy * ie;
-    const R S1 = R(6) * uF;
-    const R S7 = R(2) * (ux * Fx - uy * Fy) * ie;
-    const R S8 = (ux * Fy + uy * Fx) * ie;
-    // Lambda (m - m_eq) - (I - Lambda/2) S, component by component (S_2 = -S_1, S_4 = -F_x, ...)
-    const R d1 = c.s1 * (m1 - e1) - c.h1 * S1;
-    const R d2 = c.s2 * (m2 - e2) + c.h2 * S1;
-    const R d3 = c.s3 * (m3 - ux) - c.h3 * Fx;
-    const R d4 = c.s4 * (m4 + ux) + c.h4 * Fx;
-    const R d5 = c.s5 * (m5 - uy) - c.h5 * Fy;
-    const R d6 = c.s6 * (m6 + uy) + c.h6 * Fy;
-    const R d7 = c.s7 * (m7 - e7) - c.h7 * S7;
-    const R d8 = c.s8 * (m8 - e8) - c.h8 * S8;
-    // M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4)
-    const R a1 = d1 * R(1.0 / 36.0), a2 = d2 * R(1.0 / 36.0);
-    const R a3 = d3 * R(1.0 / 6.0), a4 = d4 * R(1.0 / 12.0);
-    const R a5 = d5 * R(1.0 / 6.0), a6 = d6 * R(1.0 / 12.0);
-    const R a7 = d7 * R(0.25), a8 = d8 * R(0.25);
-    const R axis = -a1 - R(2) * a2;
-    const R diag = R(2) * a1 + a2;
-    const R px = a3 - R(2) * a4, py = a5 - R(2) * a6;
-    const R qx = a3 + a4, qy = a5 + a6;
-    f[0] -= R(4) * (a2 - a1);
-    f[1] -= axis + px + a7;
-    f[2] -= axis + py - a7;
-    f[3] -= axis - px + a7;
-    f[4] -= axis - py - a7;
-    f[5] -= diag + qx + qy + a8;
-    f[6] -= diag - qx + qy - a8;
-    f[7] -= diag - qx - qy + a8;
-    f[8] -= diag + qx - qy - a8;
+// density moment is conserved exactly).  In that change (alpha1 = 1, alpha2 = -3, rho0 = 1)
+//   e:   m_1 - m_eq,1 = 4 fd + fa - 2 f0 - 3 u^2/eps   (rho cancels; fa, fd: the sums over the
+//   eps: m_2 - m_eq,2 = 3 (f0 - fa + u^2/eps)            axis and the diagonal populations)
+//   j:   s_3 (j_x - u_x) - (1 - s_3/2) F_x = -F_x, since u = j + F/2 (Eq. 17) is what
+//        macro() solves; the same in y
+// and a_k below is the k-th component times the factor of M^-1 = M^T diag(1/9, 1/36, 1/36,
+// 1/6, 1/12, 1/6, 1/12, 1/4, 1/4).  Opposite populations share their sums.  With the root
+// of |u| and a division gone from macro(), a node takes 179 FP64 instructions instead of
+// 250, and 170 FP32 operations.
+template <typename K, typename R>
+__device__ __forceinline__ void collide_flow(const Coef<K>& c, const Macro<R>& M, R f[9]) {
+    const R ux = M.ux, uy = M.uy, Fx = M.Fx, Fy = M.Fy;
+    const R p13 = add_(f[1], f[3]), d13 = sub_(f[1], f[3]), p24 = add_(f[2], f[4]), d24 = sub_(f[2], f[4]);
+    const R p57 = add_(f[5], f[7]), D57 = sub_(f[5], f[7]), p68 = add_(f[6], f[8]), D68 = sub_(f[6], f[8]);
+    const R fa = add_(p13, p24), fd = add_(p57, p68);
+    const R uxe = mul_(ux, R(c.inv_eps_f)), uye = mul_(uy, R(c.inv_eps_f));
+    const R A = mul_(ux, uxe), B = mul_(uy, uye);
+    const R P = mul_(uxe, Fx), Q = mul_(uye, Fy);
+    const R u2 = add_(A, B), uF = add_(P, Q);
+    const R a1 = fma_(R(c.k1), fma_(R(4), fd, fma_(R(-2), f[0], fma_(R(-3), u2, fa))), mul_(R(c.k1F), uF));
+    const R a2 = fma_(R(c.k2), sub_(add_(f[0], u2), fa), mul_(R(c.k2F), uF));
+    const R a4 = fma_(R(c.k4), fma_(R(-2), d13, add_(sub_(D57, D68), ux)), mul_(R(c.k4F), Fx));
+    const R a6 = fma_(R(c.k6), fma_(R(-2), d24, add_(add_(D57, D68), uy)), mul_(R(c.k6F), Fy));
+    const R a7 = fma_(R(c.k7), sub_(sub_(p13, A), sub_(p24, B)), mul_(R(c.k7F), sub_(P, Q)));
+    const R a8 = fma_(R(c.k8), sub_(sub_(p57, p68), mul_(ux, uye)), mul_(R(c.k8F), fma_(uxe, Fy, mul_(uye, Fx))));
+    const R gx = mul_(Fx, R(1.0 / 6.0)), gy = mul_(Fy, R(1.0 / 6.0));
+    const R ax = fma_(R(2), a2, a1), X = sub_(ax, a7), Y = add_(ax, a7);
+    const R px = fma_(R(2), a4, gx), py = fma_(R(2), a6, gy);
+    const R dg = fma_(R(2), a1, a2), U = add_(dg, a8), V = sub_(dg, a8);
+    const R qx = sub_(gx, a4), qy = sub_(gy, a6), r = add_(qx, qy), t = sub_(qx, qy);
+    f[0] = fma_(R(4), sub_(a1, a2), f[0]);
+    f[1] = add_(f[1], add_(X, px));
+    f[2] = add_(f[2], add_(Y, py));
+    f[3] = add_(f[3], sub_(X, px));
+    f[4] = add_(f[4], sub_(Y, py));
+    f[5] = add_(f[5], sub_(r, U));
+    f[6] = sub_(f[6], add_(V, t));
+    f[7] = sub_(f[7], add_(U, r));
+    f[8] = add_(f[8], sub_(t, V));
 }
 
 // The two D2Q5 collisions of a node (Eqs. 21-22) with the source of Eq. 27; hist is
 // read and updated.
-template <typename R>
-__device__ __forceinline__ void collide_scalars(const Coef<R>& c, const Macro<R>& M, R g[5], R h[5],
+template <typename K, typename R>
+__device__ __forceinline__ void collide_scalars(const Coef<K>& c, const Macro<R>& M, R g[5], R h[5],
                                                 R hist[4]) {
-    const R ux = M.ux, uy = M.uy;
     // Eq. 27 with d(Phi u)/dt = (Phi u)|t - (Phi u)|t-1 (Sec. 3.2)
-    const R T = c.T0 + M.Tp, C = c.C0 + M.Cp;
-    const R Tux = T * ux, Tuy = T * uy, Cux = C * ux, Cuy = C * uy;
-    const R XTx = Tux - hist[0], XTy = Tuy - hist[1], XCx = Cux - hist[2], XCy = Cuy - hist[3];
+    const R T = add_(R(c.T0), M.Tp), C = add_(R(c.C0), M.Cp);
+    const R Tux = mul_(T, M.ux), Tuy = mul_(T, M.uy), Cux = mul_(C, M.ux), Cuy = mul_(C, M.uy);
+    collide_d2q5(g, M.Tp, Tux, Tuy, sub_(Tux, hist[0]), sub_(Tuy, hist[1]), c.zs, c.nc3T);
+    collide_d2q5(h, M.Cp, Cux, Cuy, sub_(Cux, hist[2]), sub_(Cuy, hist[3]), c.es, c.nc3C);
     hist[0] = Tux;
     hist[1] = Tuy;
     hist[2] = Cux;
     hist[3] = Cuy;
-    collide_d2q5(g, M.Tp, T, ux, uy, XTx, XTy, c.za1, c.za2, c.za3, c.za4, c.c3T, c.hz1, c.hz2);
-    collide_d2q5(h, M.Cp, C, ux, uy, XCx, XCy, c.ed1, c.ed2, c.ed3, c.ed4, c.c3C, c.he1, c.he2);
 }
 
-template <typename R>
-__device__ __forceinline__ void collide(const Coef<R>& c, R f[9], R g[5], R h[5], R hist[4]) {
-    const Macro<R> M = macro(c, f, g, h);
+template <bool FLAT = false, typename K, typename R>
+__device__ __forceinline__ void collide(const Coef<K>& c, R f[9], R g[5], R h[5], R hist[4]) {
+    const Macro<R> M = macro<FLAT>(c, f, g, h);
     collide_flow(c, M, f);
     collide_scalars(c, M, g, h, hist);
 }

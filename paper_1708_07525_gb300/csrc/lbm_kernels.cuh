@@ -67,7 +67,8 @@ __device__ __forceinline__ int link_side(int ti, int tj, const Geom& G) {
 // no-slip rule is u_w = 0).
 template <typename R>
 __device__ __forceinline__ R wall_momentum(const Coef<R>& c, int side, int q) {
-    return R(w9_of(q)) * (R(ex_of(q)) * c.wmom[side][0] + R(ey_of(q)) * c.wmom[side][1]);
+    // e_q's components are 0 and +-1: one sum at most, and one product
+    return mul_(R(w9_of(q)), fma_(R(ex_of(q)), c.wmom[side][0], mul_(R(ey_of(q)), c.wmom[side][1])));
 }
 
 // Pre-collision populations of node (i, j) at level t from a buffer of level
@@ -127,7 +128,7 @@ __device__ __forceinline__ void gather_pull(const S* __restrict__ buf, const Geo
             const S* p = in ? buf + (size_t)(QF + slot_src) * G.plane + (size_t)sj * G.pitch + si
                             : buf + (size_t)(QF + slot_self) * G.plane + self;
             f[q] = Store<S>::ld(p);   // halfway bounce-back when !in
-            if (EXT && !in && c.moving) f[q] += wall_momentum(c, link_side(si, sj, G), q);
+            if (EXT && !in && c.moving) f[q] = add_(f[q], wall_momentum(c, link_side(si, sj, G), q));
         }
     }
 #pragma unroll
@@ -335,7 +336,7 @@ __device__ __forceinline__ void store_aa_odd(S* __restrict__ buf, const Geom& G,
         S* p = in ? buf + (size_t)(QF + q) * G.plane + (size_t)tj * G.pitch + ti
                   : buf + (size_t)(QF + opp_of(q)) * G.plane + self;
         R v = f[q];
-        if (EXT && !in && c.moving) v -= wall_momentum(c, link_side(ti, tj, G), q);
+        if (EXT && !in && c.moving) v = sub_(v, wall_momentum(c, link_side(ti, tj, G), q));
         put(p, v, sr, seed, q);
     }
 #pragma unroll
@@ -826,13 +827,6 @@ __device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-// FP32 maxima stay in FP32: GB300's FP64 pipe is narrow, and a per-block max in
-// FP64 (shuffle + fmax per step) made the residual pass FP64-bound.
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -872,11 +866,9 @@ nush_kernel(const S* __restrict__ buf, Geom G, Coef<typename Real<S>::type> c, i
             const int i = LR ? d : j, jj = LR ? j : d;
             R f[9], g[5], h[5];
             gather<false>(mode, buf, G, i, jj, c, f, g, h);
-            const R sg = ((g[0] + g[1]) + (g[2] + g[3])) + g[4];
-            const R sh = ((h[0] + h[1]) + (h[2] + h[3])) + h[4];
             const R ie = c.poro ? R(1) / c.poro[(size_t)jj * G.pitch + i] : c.inv_eps;
-            T[k] = W.T0 + (double)(sg * c.inv_sigma);
-            C[k] = W.C0 + (double)(sh * ie);
+            T[k] = W.T0 + (double)mul_(sum5(g), c.inv_sigma);
+            C[k] = W.C0 + (double)mul_(sum5(h), ie);
         }
         // inward gradient at the wall: nodes on the walls (-3 Phi_0 + 4 Phi_1 - Phi_2) / 2,
         // trapezoidal mean over the spacings along the wall; halfway walls

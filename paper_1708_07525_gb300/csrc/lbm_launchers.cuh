@@ -97,7 +97,7 @@ cudaError_t launch_step_ab(const void* src, void* dst, void* hist, const Geom& G
             // inner column pairs two nodes per thread, the edge set one node per thread,
             // in one programmatic dependent launch
             return launch_pdl(step_ab_pair_kernel<S>, gp, dim3(PAIR_BX, PAIR_BY), L.stream, (const S*)src,
-                              (S*)dst, (float*)hist, G, *L.pair, c, erows);
+                              (S*)dst, (float*)hist, G, c, erows);
     }
     if constexpr (std::is_same<R, float>::value && LBM_AB_NEE_FUSED) {
         if (c.nee) {
@@ -173,9 +173,9 @@ cudaError_t launch_step_aa(void* buf, void* hist, const Geom& G,
             const dim3 pb(PAIR_BX, PAIR_BY);
             if (!odd)
                 return launch_pdl(step_aa_even_pair_kernel<S>, ge, pb, L.stream, (S*)buf, (float*)hist, G,
-                                  *L.pair);
+                                  c);
             return launch_pdl(step_aa_odd_pair_kernel<S>, gp, pb, L.stream, (S*)buf, (float*)hist, G,
-                              *L.pair, c, erows);
+                              c, erows);
         }
     }
     const long long split_min = std::is_same<R, double>::value ? 0 : LBM_AA_SPLIT_MIN_NODES;

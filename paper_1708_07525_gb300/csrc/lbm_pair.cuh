@@ -280,6 +280,15 @@ __device__ __forceinline__ void aa_odd_edge_node(S* __restrict__ buf, float* __r
     store_hist(hist, G, self, hv);
 }
 
+// Placed between a pair's loads and its collision: a branch that is never taken (rows hold
+// at least three nodes) and that the compiler cannot see through, so that the loads end a
+// basic block and all go out before the arithmetic.
+__device__ __forceinline__ bool loads_first(const Geom& G) {
+    int n;
+    asm volatile("mov.b32 %0, %1;" : "=r"(n) : "r"(G.nx) : "memory");
+    return n > 0;
+}
+
 // ---- kernels -------------------------------------------------------------------------
 // Two-buffer pull step: block (PAIR_BX, PAIR_BY) over (1 + pairs, erows + rows 1 .. ny - 2):
 // the edge blocks (edge_index), then the inner column pairs, the first thread of a row idle
@@ -310,12 +319,12 @@ constexpr int PAIR_BX = LBM_PAIR_BX, PAIR_BY = LBM_PAIR_BY;
 template <typename S>
 __global__ void __launch_bounds__(PAIR_BX * PAIR_BY, LBM_PAIR_MIN_BLOCKS)
 step_ab_pair_kernel(const S* __restrict__ src, S* __restrict__ dst, float* __restrict__ hist, Geom G,
-                    Coef<f2> c, Coef<float> c1, int erows) {
+                    Coef<float> c, int erows) {
     pdl_trigger();
     pdl_wait();                                // launched by launch_pdl()
     if ((int)blockIdx.y < erows) {
         const long long k = edge_index();
-        if (k < edge_count(G)) ab_edge_node(src, dst, hist, G, c1, k);
+        if (k < edge_count(G)) ab_edge_node(src, dst, hist, G, c, k);
         return;
     }
     int m, j;
@@ -324,6 +333,7 @@ step_ab_pair_kernel(const S* __restrict__ src, S* __restrict__ dst, float* __res
     f2 f[9], g[5], h[5], hv[4];
     gather_pair_pull<false, LBM_PAIR_AB_NC>(src, G, self, f, g, h);
     load_hist_pair(hist, G, self, hv);
+    if (!loads_first(G)) return;
     uint32_t state = pair_seed(self, f[0], g[0]);
     const Macro<f2> M = macro(c, f, g, h);
     collide_flow(c, M, f);
@@ -337,7 +347,7 @@ step_ab_pair_kernel(const S* __restrict__ src, S* __restrict__ dst, float* __res
 // (nx / 2, ny).
 template <typename S>
 __global__ void __launch_bounds__(PAIR_BX * PAIR_BY, LBM_PAIR_MIN_BLOCKS)
-step_aa_even_pair_kernel(S* __restrict__ buf, float* __restrict__ hist, Geom G, Coef<f2> c) {
+step_aa_even_pair_kernel(S* __restrict__ buf, float* __restrict__ hist, Geom G, Coef<float> c) {
     pdl_trigger();
     pdl_wait();                                // launched by launch_pdl()
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -347,6 +357,7 @@ step_aa_even_pair_kernel(S* __restrict__ buf, float* __restrict__ hist, Geom G, 
     f2 f[9], g[5], h[5], hv[4];
     gather_pair_local(buf, G, self, f, g, h);
     load_hist_pair(hist, G, self, hv);
+    if (!loads_first(G)) return;
     uint32_t state = pair_seed(self, f[0], g[0]);
     const Macro<f2> M = macro(c, f, g, h);
     collide_flow(c, M, f);
@@ -360,13 +371,13 @@ step_aa_even_pair_kernel(S* __restrict__ buf, float* __restrict__ hist, Geom G, 
 // writes only its own node's or pair's locations, so the two parts touch disjoint memory).
 template <typename S>
 __global__ void __launch_bounds__(PAIR_BX * PAIR_BY, LBM_PAIR_MIN_BLOCKS)
-step_aa_odd_pair_kernel(S* __restrict__ buf, float* __restrict__ hist, Geom G, Coef<f2> c,
-                        Coef<float> c1, int erows) {
+step_aa_odd_pair_kernel(S* __restrict__ buf, float* __restrict__ hist, Geom G, Coef<float> c,
+                        int erows) {
     pdl_trigger();
     pdl_wait();                                // launched by launch_pdl()
     if ((int)blockIdx.y < erows) {
         const long long k = edge_index();
-        if (k < edge_count(G)) aa_odd_edge_node(buf, hist, G, c1, k);
+        if (k < edge_count(G)) aa_odd_edge_node(buf, hist, G, c, k);
         return;
     }
     int m, j;
@@ -375,6 +386,7 @@ step_aa_odd_pair_kernel(S* __restrict__ buf, float* __restrict__ hist, Geom G, C
     f2 f[9], g[5], h[5], hv[4];
     gather_pair_pull<true, true>(buf, G, self, f, g, h);
     load_hist_pair(hist, G, self, hv);
+    if (!loads_first(G)) return;
     uint32_t state = pair_seed(self, f[0], g[0]);
     const Macro<f2> M = macro(c, f, g, h);
     collide_flow(c, M, f);
