@@ -90,8 +90,10 @@ typedef struct {
     lbm_alloc_fn alloc;         /* NULL -> cudaMalloc / cudaFree */
     lbm_free_fn free;
     void* alloc_user;
-    int block_x, block_y;       /* launch tile of the step kernel: block_x a multiple of 32,
-                                   block_x * block_y <= 256; 0 -> tuned default */
+    int block_x, block_y;       /* launch tile of the one-step kernels: block_x a multiple of 32,
+                                   block_x * block_y <= 256; 0 -> tuned default (and two
+                                   steps per launch where that is faster: FP32, two buffers,
+                                   halfway walls, from 750,000 nodes on) */
     int graph_chunk;            /* steps per captured CUDA graph; 0 -> default, <0 -> off */
     const double* eps_field;    /* optional host [ny][nx] porosity field: the REV model with
                                    spatially varying eps (Sec. 2-3 applied per node, F_eps of
@@ -221,7 +223,8 @@ lbm_status lbm_create_raw(const lbm_params* params, const lbm_options* opt, lbm_
 lbm_status lbm_reset(lbm_ctx* ctx, const double* T_init, const double* C_init, uint64_t seed,
                      double noise);
 
-/* Advance n >= 0 time steps (asynchronous on the context's stream).  On a stream other
+/* Advance n >= 0 time steps (asynchronous on the context's stream).  The result does not
+ * depend on how n steps are split over calls.  On a stream other
  * than the legacy default stream the steps are replayed from CUDA graphs in chunks, and
  * a step that is one kernel goes out as a programmatic dependent launch: its blocks may
  * be placed while the kernel before it on the stream drains, but each waits for that

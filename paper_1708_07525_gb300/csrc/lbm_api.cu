@@ -175,7 +175,9 @@ struct lbm_ctx {
     Geom G{};
     size_t esz = 8, rsz = 8;
     void* buf[2] = {nullptr, nullptr};
-    void* hist = nullptr;
+    void* hist = nullptr;           // history of the current level
+    void* hist_alt = nullptr;       // second history buffer (two steps per launch), or NULL
+    int hcur = 0;                   // swaps of hist and hist_alt so far, mod 2
     double* d_out = nullptr;        // OUT_DOUBLES: Nu/Sh and residual results, Nu/Sh partial sums
     double* d_fields = nullptr;     // lazily allocated [5][h][w] read-out window
     size_t fields_cap = 0;          // nodes d_fields holds
@@ -198,7 +200,9 @@ struct lbm_ctx {
     LaunchCfg L{};
     int graph_chunk = 0;
     bool round_nearest = false;     // 16-bit storage: nearest-even instead of stochastic
-    cudaGraphExec_t graph = nullptr;
+    // captured chunks by the buffers they start from: [2 * cur + hcur]
+    cudaGraphExec_t graph[4] = {nullptr, nullptr, nullptr, nullptr};
+    int graph_end[4] = {0, 0, 0, 0};   // and the buffers they end on
     lbm_alloc_fn alloc = nullptr;
     lbm_free_fn free_fn = nullptr;
     void* alloc_user = nullptr;
@@ -278,6 +282,35 @@ cudaError_t one_step(lbm_ctx* c) {
         default: e = dispatch_step<__half>(c); break;
     }
     c->t += 1;
+    return e;
+}
+
+// Two steps in one launch (lbm_march.cuh): FP32, two buffers, halfway walls, a second
+// history buffer, which only cavities that take them have.
+bool can_march(const lbm_ctx* c) { return c->hist_alt != nullptr && !c->P.nee; }
+
+cudaError_t two_steps(lbm_ctx* c) {
+    cudaError_t e = launch_step2_ab(c->buf[c->cur], c->buf[c->cur ^ 1], c->hist, c->hist_alt, c->G, c->cf, c->L);
+    c->cur ^= 1;
+    std::swap(c->hist, c->hist_alt);
+    c->hcur ^= 1;
+    c->t += 2;
+    return e;
+}
+
+// Enqueues n steps; stops at the first error.
+cudaError_t enqueue(lbm_ctx* c, int64_t n) {
+    cudaError_t e = cudaSuccess;
+    const bool march = can_march(c);
+    while (n > 0 && e == cudaSuccess) {
+        if (march && n >= 2) {
+            e = two_steps(c);
+            n -= 2;
+        } else {
+            e = one_step(c);
+            n -= 1;
+        }
+    }
     return e;
 }
 
@@ -672,6 +705,15 @@ lbm_status create_core(const lbm_params* params, const lbm_options* opt, int sla
     c->buf[0] = c->dalloc(c->state_bytes());
     if (c->layout == LBM_AB_PULL) c->buf[1] = c->dalloc(c->state_bytes());
     c->hist = c->dalloc(c->hist_bytes());
+    if (c->prec == LBM_F32 && c->layout == LBM_AB_PULL && !slab && !O.eps_field && !O.K_field && !O.block_x &&
+        !O.block_y && march_fits(c->G)) {
+        // two steps per launch write a second history buffer; without it (no memory for it, or
+        // a state of more than a quarter of the device, which leaves the rest to the
+        // caller) every step is a launch
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && 2 * c->state_bytes() < total_b / 4)
+            c->hist_alt = c->dalloc(c->hist_bytes());
+    }
     c->d_out = (double*)c->dalloc(OUT_DOUBLES * sizeof(double));
     if (O.eps_field || O.K_field) {
         if (c->P.model_a) {
@@ -734,6 +776,7 @@ lbm_status create_core(const lbm_params* params, const lbm_options* opt, int sla
     cudaMemsetAsync(c->buf[0], 0, c->state_bytes(), c->stream);
     if (c->buf[1]) cudaMemsetAsync(c->buf[1], 0, c->state_bytes(), c->stream);
     cudaMemsetAsync(c->hist, 0, c->hist_bytes(), c->stream);
+    if (c->hist_alt) cudaMemsetAsync(c->hist_alt, 0, c->hist_bytes(), c->stream);
     cudaMemsetAsync(c->d_out, 0, OUT_DOUBLES * sizeof(double), c->stream);   // the block count of the Nu/Sh pass
 
     if ((O.T_init == nullptr) != (O.C_init == nullptr)) {
@@ -797,42 +840,54 @@ lbm_status lbm_step(lbm_ctx* c, int64_t n) {
     }
     DeviceGuard dg(c->device);
     cudaError_t e = cudaSuccess;
-    // Graph replay needs the even-parity state the graph was captured from.
-    while (n > 0 && (c->t & 1) && e == cudaSuccess) {
+    // the in-place layout replays its graph from even levels
+    while (n > 0 && c->layout == LBM_AA && (c->t & 1) && e == cudaSuccess) {
         e = one_step(c);
         --n;
     }
     if (c->graph_chunk > 0 && n >= c->graph_chunk && e == cudaSuccess) {
-        if (!c->graph) {
-            cudaGraph_t g = nullptr;
-            e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
-            if (e == cudaSuccess) {
-                const int64_t t0 = c->t;
-                const int cur0 = c->cur;
-                cudaError_t le = cudaSuccess;
-                for (int k = 0; k < c->graph_chunk && le == cudaSuccess; ++k) le = one_step(c);
-                c->t = t0;   // capture records, it does not run
-                c->cur = cur0;
-                e = cudaStreamEndCapture(c->stream, &g);
-                if (le != cudaSuccess) e = le;
-            }
-            if (e == cudaSuccess) e = cudaGraphInstantiate(&c->graph, g, 0);
-            if (g) cudaGraphDestroy(g);
-            if (e != cudaSuccess) {
-                c->graph = nullptr;
-                return c->cuda_fail(e, "lbm_step: graph capture");
-            }
-        }
         while (n >= c->graph_chunk && e == cudaSuccess) {
-            e = cudaGraphLaunch(c->graph, c->stream);
-            c->t += c->graph_chunk;   // even chunk: buffer parity unchanged
-            n -= c->graph_chunk;
+            // a chunk is captured once per pair of buffers it can start from, and may end
+            // on the others
+            const int k0 = 2 * c->cur + c->hcur;
+            const int64_t t0 = c->t;
+            if (!c->graph[k0]) {
+                const int cur0 = c->cur, hcur0 = c->hcur;
+                void *h0 = c->hist, *h1 = c->hist_alt;
+                cudaGraph_t g = nullptr;
+                e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
+                if (e == cudaSuccess) {
+                    const cudaError_t le = enqueue(c, c->graph_chunk);
+                    c->t = t0;   // capture records, it does not run
+                    c->graph_end[k0] = 2 * c->cur + c->hcur;
+                    c->cur = cur0;
+                    c->hcur = hcur0;
+                    c->hist = h0;
+                    c->hist_alt = h1;
+                    e = cudaStreamEndCapture(c->stream, &g);
+                    if (le != cudaSuccess) e = le;
+                }
+                if (e == cudaSuccess) e = cudaGraphInstantiate(&c->graph[k0], g, 0);
+                if (g) cudaGraphDestroy(g);
+                if (e != cudaSuccess) {
+                    c->graph[k0] = nullptr;
+                    return c->cuda_fail(e, "lbm_step: graph capture");
+                }
+            }
+            e = cudaGraphLaunch(c->graph[k0], c->stream);
+            if (e == cudaSuccess) {
+                const int k1 = c->graph_end[k0];
+                c->cur = k1 >> 1;
+                if ((k1 & 1) != c->hcur) {
+                    std::swap(c->hist, c->hist_alt);
+                    c->hcur ^= 1;
+                }
+                c->t += c->graph_chunk;
+                n -= c->graph_chunk;
+            }
         }
     }
-    while (n > 0 && e == cudaSuccess) {
-        e = one_step(c);
-        --n;
-    }
+    if (e == cudaSuccess) e = enqueue(c, n);
     if (e != cudaSuccess) return c->cuda_fail(e, "lbm_step");
     return LBM_OK;
 }
@@ -1161,7 +1216,7 @@ lbm_status lbm_load(lbm_ctx* c, const void* buf, size_t len) {
     if (h.pitch < h.nx || len < sizeof h + src_state + src_hist)
         return c->fail(LBM_ERR_INVALID, "lbm_load: truncated checkpoint");
     DeviceGuard dg(c->device);
-    // the two-buffer layout keeps the state in buffer (t mod 2), which the captured graph relies on
+    // the two-buffer layout starts again in buffer (t mod 2)
     const int slot = c->layout == LBM_AB_PULL ? (int)(h.t & 1) : 0;
     const char* p = (const char*)buf + sizeof h;
     cudaError_t e;
@@ -1215,9 +1270,9 @@ lbm_status lbm_load(lbm_ctx* c, const void* buf, size_t len) {
     c->cf.seed_off = (long long)(c->slab_y0 - c->G.jb) * c->G.pitch;
     c->cd.poro = (c->poro && c->rsz == 8) ? (const double*)c->poro : nullptr;
     c->cf.poro = (c->poro && c->rsz == 4) ? (const float*)c->poro : nullptr;
-    if (c->graph) {   // constants are baked into the captured launches
-        cudaGraphExecDestroy(c->graph);
-        c->graph = nullptr;
+    for (cudaGraphExec_t& g : c->graph) {   // constants are baked into the captured launches
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
     }
     c->t = h.t;
     c->cur = slot;
@@ -1240,10 +1295,12 @@ void lbm_destroy(lbm_ctx* c) {
     if (!c) return;
     DeviceGuard dg(c->device);
     if (c->stream) cudaStreamSynchronize(c->stream);
-    if (c->graph) cudaGraphExecDestroy(c->graph);
+    for (cudaGraphExec_t g : c->graph)
+        if (g) cudaGraphExecDestroy(g);
     c->dfree(c->buf[0], c->state_bytes());
     c->dfree(c->buf[1], c->state_bytes());
     c->dfree(c->hist, c->hist_bytes());
+    c->dfree(c->hist_alt, c->hist_bytes());
     c->dfree(c->d_out, OUT_DOUBLES * sizeof(double));
     c->dfree(c->d_fields, 5 * c->fields_cap * sizeof(double));
     c->dfree(c->d_snap, 4 * c->nodes() * c->rsz);

@@ -94,6 +94,11 @@ cudaError_t launch_step_ab(const void* src, void* dst, void* hist, const Geom& G
 template <typename S>
 cudaError_t launch_step_aa(void* buf, void* hist, const Geom& G,
                            const Coef<typename Real<S>::type>& c, bool odd, const LaunchCfg& L);
+// Two steps of the FP32 two-buffer layout with halfway walls in one launch, from the history
+// hist to hist_out (lbm_march.cuh).
+cudaError_t launch_step2_ab(const void* src, void* dst, const void* hist, void* hist_out, const Geom& G,
+                            const Coef<float>& c, const LaunchCfg& L);
+bool march_fits(const Geom& G);
 // Fields over the window [x0, x0 + w) x [y0, y0 + h) into out[5][h][w].
 template <typename S>
 cudaError_t launch_fields(const void* buf, const Geom& G, const Coef<typename Real<S>::type>& c,
