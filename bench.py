@@ -35,7 +35,8 @@ BYTES_PER_NODE_19 = {"f64": 2 * 19 * 8, "f32": 2 * 19 * 4, "bf16": 2 * 19 * 2, "
 KERNEL_SOURCES = ["paper_1708_07525_gb300/csrc/lbm_kernels.cuh",
                   "paper_1708_07525_gb300/csrc/lbm_device.cuh",
                   "paper_1708_07525_gb300/csrc/lbm_launchers.cuh",
-                  "paper_1708_07525_gb300/csrc/lbm_march.cuh"]
+                  "paper_1708_07525_gb300/csrc/lbm_march.cuh",
+                  "paper_1708_07525_gb300/csrc/lbm_fixed.cuh"]
 
 
 def kernel_hash() -> str:
@@ -220,18 +221,10 @@ def steps_per_launch(args):
 
 def step_launches(args, k):
     """Kernels launched by k time steps of the benchmark cavity: half as many where a launch
-    takes two steps (steps_per_launch; an odd step is one of its own).  With FP32 arithmetic
-    (FP32 and 16-bit storage) every step is one launch: the FP32 steps, the in-place odd
-    step with its ring in the same launch, the step with wall nodes with its wall ring in
-    the same launch, the 16-bit pair steps with their edge set.  FP64 splits the two-buffer
-    step (also with wall nodes) and the in-place odd step into an inner-node launch and a
-    ring launch on a second stream."""
-    if args.precision != "f64":
-        per = steps_per_launch(args)
-        return k // per + k % per
-    if args.layout == "aa":
-        return k + k // 2
-    return 2 * k
+    takes two steps (steps_per_launch; an odd step is one of its own).  Every other step is
+    one launch, walls included, in every precision and layout."""
+    per = steps_per_launch(args)
+    return k // per + k % per
 
 
 def run_ours(args):
@@ -353,7 +346,7 @@ def run_ours(args):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "peak_source": f"{peak_kind} hbm_gbs",
-                     "kernel": ((f"step_ab_kernel<{args.precision}> (inner nodes) + nee_ring_kernel"
+                     "kernel": (("step_ab_nee_flat_kernel (FP64)"
                                  if args.precision == "f64" else
                                  f"step_ab_nee_fused_kernel<{args.precision}> (wall ring and inner "
                                  f"nodes in one launch)")
@@ -364,6 +357,8 @@ def run_ours(args):
                                       if args.precision in ("bf16", "f16")
                                       else "step2_ab_kernel (two time steps per launch)"
                                       if per == 2
+                                      else f"step_{args.layout}_flat_kernel (FP64)"
+                                      if args.precision == "f64"
                                       else f"step_{args.layout}_kernel<{args.precision}>")),
                      "kernel_us_per_launch": launch_ms * 1e3,
                      "time_steps_per_launch": per,

@@ -41,6 +41,70 @@ size_t storage_size(int prec) {
 }  // namespace
 
 namespace lbm {
+namespace {
+template <int B>
+void set_const(FxConst<B>& k, long double c) {
+    k.c = (unsigned long long)llrintl(ldexpl(fabsl(c), 63 + B)) & ~1ull;
+}
+// What fx_plus / fx_minus / fx_one take off: half the constants (the offset of the products'
+// arguments) less the rounding of quarters, which makes up for the floors of a sum (two
+// quarters' halves down), of a difference (none) or of one product.
+template <int B, int D>
+long long less_plus(FxConst<B> c, FxConst<D> d) { return (long long)(c.c / 2 + d.c / 2) - 2; }
+template <int B, int D>
+long long less_minus(FxConst<B> c, FxConst<D> d) { return (long long)(c.c / 2 - d.c / 2) - 1; }
+template <int B>
+long long less_one(FxConst<B> c) { return (long long)(c.c / 2) - 2; }
+
+FixedScalar fixed_scalar(const double r[5], long double nc3_over_cap) {
+    FixedScalar k;
+    set_const(k.b1, 0.5L * r[1]);
+    set_const(k.q1, 0.5L - 0.25L * r[1]);
+    set_const(k.b2, 0.5L * r[2]);
+    set_const(k.q2, 0.5L - 0.25L * r[2]);
+    set_const(k.b3, r[3] / 20.0L);
+    set_const(k.b4, 0.25L * r[4]);
+    set_const(k.p, r[3] / 20.0L * nc3_over_cap);
+    k.p_neg = nc3_over_cap < 0.0L;
+    k.less1 = less_minus(k.b1, k.q1);
+    k.less2 = less_minus(k.b2, k.q2);
+    k.less3 = less_plus(k.b3, k.p);
+    k.less4 = less_one(k.b4);
+    return k;
+}
+void set_fixed(NoFixed&, const lbm_params&) {}
+void set_fixed(FixedCoef& k, const lbm_params& P) {
+    // the rates lie in (0, 2), which bounds every factor but the last one's
+    const long double pT = P.model_a ? 4.0L - 5.0L * P.varpi : 4.0L - 5.0L * P.varpi / P.sigma;
+    const long double pC = P.model_a ? 4.0L - 5.0L * P.varpi : 4.0L - 5.0L * P.varpi / P.eps;
+    k.on = fabsl(pT * P.zeta[3] / 20.0L) < 1.0L && fabsl(pC * P.eta[3] / 20.0L) < 1.0L;
+    if (!k.on) return;
+    auto h = [](double s) { return 1.0L - 0.5L * s; };
+    set_const(k.k1, P.s[1] / 36.0L);
+    set_const(k.k1F, h(P.s[1]) / 6.0L);
+    set_const(k.k2, P.s[2] / 12.0L);
+    set_const(k.k2F, h(P.s[2]) / 6.0L);
+    set_const(k.k4, P.s[4] / 12.0L);
+    set_const(k.k4F, h(P.s[4]) / 12.0L);
+    set_const(k.k6, P.s[6] / 12.0L);
+    set_const(k.k6F, h(P.s[6]) / 12.0L);
+    set_const(k.k7, P.s[7] / 4.0L);
+    set_const(k.k7F, h(P.s[7]) / 2.0L);
+    set_const(k.k8, P.s[8] / 4.0L);
+    set_const(k.k8F, h(P.s[8]) / 4.0L);
+    set_const(k.sixth, 1.0L / 6.0L);
+    k.less1 = less_minus(k.k1, k.k1F);
+    k.less2 = less_plus(k.k2, k.k2F);
+    k.less4 = less_plus(k.k4, k.k4F);
+    k.less6 = less_plus(k.k6, k.k6F);
+    k.less7 = less_minus(k.k7, k.k7F);
+    k.less8 = less_minus(k.k8, k.k8F);
+    k.less_sixth = less_one(k.sixth);
+    k.zs = fixed_scalar(P.zeta, pT);
+    k.es = fixed_scalar(P.eta, pC);
+}
+}  // namespace
+
 template <typename R>
 Coef<R> make_coef(const lbm_params& P) {
     Coef<R> c;
@@ -125,6 +189,7 @@ Coef<R> make_coef(const lbm_params& P) {
     c.aT1 = (R)(P.sigma / 5.0 + c3T / 20.0);
     c.aC0 = (R)((eps - c3C) / 5.0);
     c.aC1 = (R)(eps / 5.0 + c3C / 20.0);
+    set_fixed(c.fx, P);
     return c;
 }
 template Coef<float> make_coef<float>(const lbm_params&);

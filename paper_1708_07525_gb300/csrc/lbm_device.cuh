@@ -244,6 +244,32 @@ template <typename S> struct Real { using type = float; };
 template <> struct Real<double> { using type = double; };
 
 // ---- per-instance constants (prepared on the host, passed by value) ------------
+// The constants of the integer form of the FP64 collision (lbm_fixed.cuh).
+// A positive constant c < 2^-B as the even integer c 2^(63 + B); fx_pair() and fx_one() shift their
+// arguments by the other 3 - B bits.  `less` (of a pair or a lone constant) takes off what
+// their offset-binary products hold too much, and adds the rounding.
+template <int B> struct FxConst { unsigned long long c; };
+struct FixedScalar {
+    FxConst<0> b1, q1, b2, q2, p;   // r_1 / 2, (1 - r_1 / 2) / 2 and the same for r_2; the factor of
+                                    // the scalar's sum in the third moment, |r_3 nc3 / (20 cap)|
+    FxConst<3> b3;                  // r_3 / 20
+    FxConst<1> b4;                  // r_4 / 4
+    long long less1, less2, less3, less4;
+    int p_neg;                      // the sign of p's factor
+};
+struct FixedCoef {
+    int on;                         // 0: p's factor does not lie below 1 (extreme varpi / cap), FP64 instead
+    FxConst<3> k1, k4F, k6F;
+    FxConst<2> k1F, k2, k2F, k4, k6, k8F, sixth;
+    FxConst<1> k7, k7F, k8;
+    long long less1, less2, less4, less6, less7, less8, less_sixth;
+    FixedScalar zs, es;
+};
+
+struct NoFixed {};
+template <typename R> struct FixedOf { using type = NoFixed; };
+template <> struct FixedOf<double> { using type = FixedCoef; };
+
 template <typename R>
 struct CoefScalar {
     R b1, q1, b2, q2, b3, b4;
@@ -292,6 +318,7 @@ struct Coef {
     R bT[4], bC[4];
     R uwall[4][2];
     R aT0, aT1, aC0, aC1;
+    typename FixedOf<R>::type fx;
 };
 
 
@@ -317,6 +344,7 @@ __device__ __forceinline__ void porous_at(Coef<R>& c, size_t self, size_t plane)
     c.nc3C = R(4) * e - c.varpi5;
     c.aC0 = (e + c.nc3C) * R(0.2);
     c.aC1 = e * R(0.2) - c.nc3C * R(0.05);
+    if constexpr (std::is_same<R, double>::value) c.fx.on = 0;   // its constants are the uniform medium's
 }
 
 // Macroscopic quantities of one node from pre-collision deviations.
@@ -441,8 +469,18 @@ __device__ __forceinline__ void collide_scalars(const Coef<K>& c, const Macro<R>
     hist[3] = Cuy;
 }
 
+}  // namespace lbm
+#include "lbm_fixed.cuh"
+namespace lbm {
+
 template <bool FLAT = false, typename K, typename R>
 __device__ __forceinline__ void collide(const Coef<K>& c, R f[9], R g[5], R h[5], R hist[4]) {
+    if constexpr (std::is_same<R, double>::value) {
+        if (c.fx.on) {
+            collide_fixed(c, f, g, h, hist);
+            return;
+        }
+    }
     const Macro<R> M = macro<FLAT>(c, f, g, h);
     collide_flow(c, M, f);
     collide_scalars(c, M, g, h, hist);

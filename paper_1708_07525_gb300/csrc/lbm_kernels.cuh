@@ -179,9 +179,13 @@ __device__ __forceinline__ R nee_scalar(const Coef<R>& c, int di, int dj, const 
     if (di && b[sv] == R(0) && ((c.dirichlet_mask >> sv) & 1)) return Pw[sv];
     if (dj && b[sh] == R(0) && ((c.dirichlet_mask >> sh) & 1)) return Pw[sh];
     R a = R(0), w = R(0);
-    if (di) { a += b[sv]; w += b[sv] * Pw[sv]; }
-    if (dj) { a += b[sh]; w += b[sh] * Pw[sh]; }
-    return (R(4) * Pf - Pff + R(2) * w) / (R(3) + R(2) * a);
+    if (di) { a = add_(a, b[sv]); w = fma_(b[sv], Pw[sv], w); }
+    if (dj) { a = add_(a, b[sh]); w = fma_(b[sh], Pw[sh], w); }
+    const R num = fma_(R(2), w, fma_(R(4), Pf, -Pff)), den = fma_(R(2), a, R(3));
+    if (sizeof(R) == 4) return num / den;
+    // FP64: a reciprocal and one correction by the residual
+    const R r = rcp_pos<false>(den), q = mul_(num, r);
+    return fma_(fnma_(den, q, num), r, q);
 }
 
 // Pre-collision populations (deviations) of wall node (i, j) with inward link (di, dj)
@@ -209,32 +213,46 @@ __device__ __forceinline__ void nee_rebuild(const S* __restrict__ buf, const Geo
         inv_eps_ff = R(1) / c.poro[(size_t)(j + 2 * dj) * G.pitch + (i + 2 * di)];
     }
     const Macro<R> M = macro(cf, f, g, h);
-    const R Tff = (((g2[0] + g2[1]) + (g2[2] + g2[3])) + g2[4]) * c.inv_sigma;   // Eq. 26
-    const R Cff = (((h2[0] + h2[1]) + (h2[2] + h2[3])) + h2[4]) * inv_eps_ff;
+    const R Tff = mul_(sum5(g2), c.inv_sigma);                       // Eq. 26
+    const R Cff = mul_(sum5(h2), inv_eps_ff);
     const R Tb = nee_scalar(c, di, dj, c.TwP, c.bT, M.Tp, Tff);
     const R Cb = nee_scalar(c, di, dj, c.CwP, c.bC, M.Cp, Cff);
     const int sv = dj ? (dj > 0 ? 2 : 3) : (di > 0 ? 0 : 1);
     const R ubx = c.uwall[sv][0], uby = c.uwall[sv][1];
-    const R ub2 = ubx * ubx + uby * uby, uf2 = M.ux * M.ux + M.uy * M.uy;
+    // Q(u_w) - Q(u_f) = 3 e . d + 4.5 e . A e - 1.5 tr A with d = u_w - u_f and the tensor
+    // A = u_w u_w / eps_b - u_f u_f / eps_f
     const R ieb = cb.inv_eps_f, ief = cf.inv_eps_f;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        const R eb = R(ex_of(q)) * ubx + R(ey_of(q)) * uby;
-        const R ef = R(ex_of(q)) * M.ux + R(ey_of(q)) * M.uy;
-        const R Qb = R(3) * eb + (R(4.5) * eb * eb - R(1.5) * ub2) * ieb;
-        const R Qf = R(3) * ef + (R(4.5) * ef * ef - R(1.5) * uf2) * ief;
-        f[q] += R(w9_of(q)) * (Qb - Qf);
-    }
-    const R TB = c.T0 + Tb, TF = c.T0 + M.Tp, CB = c.C0 + Cb, CF = c.C0 + M.Cp;
-    g[0] += c.aT0 * (Tb - M.Tp);
-    h[0] += cb.aC0 * Cb - cf.aC0 * M.Cp;
-#pragma unroll
-    for (int q = 1; q < 5; ++q) {
-        const R eb = R(ex_of(q)) * ubx + R(ey_of(q)) * uby;
-        const R ef = R(ex_of(q)) * M.ux + R(ey_of(q)) * M.uy;
-        g[q] += c.aT1 * (Tb - M.Tp) + R(0.5) * (eb * TB - ef * TF);
-        h[q] += cb.aC1 * Cb - cf.aC1 * M.Cp + R(0.5) * (eb * CB - ef * CF);
-    }
+    const R fex = mul_(M.ux, ief), fey = mul_(M.uy, ief), bex = mul_(ubx, ieb), bey = mul_(uby, ieb);
+    const R Axx = fma_(ubx, bex, -mul_(M.ux, fex)), Ayy = fma_(uby, bey, -mul_(M.uy, fey));
+    const R Axy = mul_(R(0.25), fma_(ubx, bey, -mul_(M.ux, fey)));
+    const R tr = add_(Axx, Ayy), diag = mul_(R(1.0 / 12.0), tr);
+    const R dx = sub_(ubx, M.ux), dy = sub_(uby, M.uy);
+    const R axx = mul_(R(1.0 / 6.0), fma_(R(3), Axx, -tr)), axy = mul_(R(1.0 / 6.0), fma_(R(3), Ayy, -tr));
+    f[0] = fma_(R(-2.0 / 3.0), tr, f[0]);
+    f[1] = add_(f[1], fma_(R(1.0 / 3.0), dx, axx));
+    f[2] = add_(f[2], fma_(R(1.0 / 3.0), dy, axy));
+    f[3] = add_(f[3], fma_(R(-1.0 / 3.0), dx, axx));
+    f[4] = add_(f[4], fma_(R(-1.0 / 3.0), dy, axy));
+    const R dp = mul_(R(1.0 / 12.0), add_(dx, dy)), dm = mul_(R(1.0 / 12.0), sub_(dx, dy));
+    f[5] = add_(f[5], add_(add_(diag, Axy), dp));
+    f[6] = add_(f[6], sub_(sub_(diag, Axy), dm));
+    f[7] = add_(f[7], sub_(add_(diag, Axy), dp));
+    f[8] = add_(f[8], add_(sub_(diag, Axy), dm));
+    const R TB = add_(c.T0, Tb), TF = add_(c.T0, M.Tp), CB = add_(c.C0, Cb), CF = add_(c.C0, M.Cp);
+    const R dT = sub_(Tb, M.Tp), gT = mul_(c.aT1, dT);
+    const R jTx = mul_(R(0.5), fma_(ubx, TB, -mul_(M.ux, TF))), jTy = mul_(R(0.5), fma_(uby, TB, -mul_(M.uy, TF)));
+    const R gC = fma_(cb.aC1, Cb, -mul_(cf.aC1, M.Cp));
+    const R jCx = mul_(R(0.5), fma_(ubx, CB, -mul_(M.ux, CF))), jCy = mul_(R(0.5), fma_(uby, CB, -mul_(M.uy, CF)));
+    g[0] = fma_(c.aT0, dT, g[0]);
+    h[0] = add_(h[0], fma_(cb.aC0, Cb, -mul_(cf.aC0, M.Cp)));
+    g[1] = add_(g[1], add_(gT, jTx));
+    g[2] = add_(g[2], add_(gT, jTy));
+    g[3] = add_(g[3], sub_(gT, jTx));
+    g[4] = add_(g[4], sub_(gT, jTy));
+    h[1] = add_(h[1], add_(gC, jCx));
+    h[2] = add_(h[2], add_(gC, jCy));
+    h[3] = add_(h[3], sub_(gC, jCx));
+    h[4] = add_(h[4], sub_(gC, jCy));
 }
 
 // Pre-collision populations of node (i, j) on a grid with wall nodes: the plain pull
@@ -410,6 +428,7 @@ step_ab_kernel(const S* __restrict__ src, S* __restrict__ dst,
     ab_node<S, EXT, INNER>(src, dst, hist, G, c, i, j);
 }
 
+__host__ __device__ inline long long ring_count(const Geom& G) { return 2LL * G.nx + 2LL * (G.ny - 2); }
 // Node k of the outermost ring, k = 0 .. 2 nx + 2 (ny - 2) - 1: bottom row, top row,
 // left column, right column (rows 1 .. ny - 2).
 __device__ __forceinline__ void ring_node(const Geom& G, long long k, int& i, int& j) {
@@ -508,6 +527,113 @@ step_ab_nee_fused_kernel(const S* __restrict__ src, S* __restrict__ dst,
     ab_node<S, EXT, true>(src, dst, hist, G, c, i, j);
 }
 
+// ---- the fused step, in-place AA layout -------------------------------------------
+// Even step (level t even): natural pre-collision values at x -> collide ->
+// post-collision value of direction q stored in slot opp(q) of x.
+// Odd step: pull from the swapped slots of the neighbours (with wall rules),
+// collide, push post-collision value of direction q into slot q of x + e_q
+// (or, where that link crosses a wall, the reflected value into slot opp(q)
+// of x).  Each thread reads and writes the same set of locations, so the
+// update is race-free in place.
+template <typename S, bool ODD, bool EXT, typename R>
+__device__ __forceinline__ void aa_node(S* __restrict__ buf, R* __restrict__ hist, const Geom& G, const Coef<R>& c,
+                                        int i, int j) {
+    R f[9], g[5], h[5], hv[4];
+    const size_t self = (size_t)j * G.pitch + i;
+    if (ODD)
+        gather_pull<true, true, EXT>(buf, G, i, j, c, f, g, h);
+    else
+        gather_local<true>(buf, G, i, j, f, g, h);
+    load_hist(hist, G, self, hv);
+    uint32_t seed = Store<S>::kLow ? node_seed(self, f[0], g[0]) : 0u;
+    collide_node<EXT>(c, self, G.plane, f, g, h, hv);
+    if (ODD)
+        store_aa_odd<EXT>(buf, G, i, j, self, c, f, g, h, seed);
+    else
+        store_aa_even(buf, G, self, c, f, g, h, seed);
+    store_hist(hist, G, self, hv);
+}
+
+template <typename S, bool ODD, bool EXT>
+__global__ void __launch_bounds__(256)
+step_aa_kernel(S* __restrict__ buf, typename Real<S>::type* __restrict__ hist, Geom G,
+               Coef<typename Real<S>::type> c) {
+    pdl_trigger();
+    pdl_wait();                                // launched by launch_pdl()
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.y * blockDim.y + threadIdx.y;
+    if (i >= G.nx || j >= G.ny) return;
+    aa_node<S, ODD, EXT>(buf, hist, G, c, i, j);
+}
+
+// FP64 steps, one thread per node in the order of storage without the padding.  A warp's
+// instruction costs the same whatever the number of its active lanes, in the FP64 pipe 64
+// clocks (see lbm_fixed.cuh), so every warp is full: 129^2 nodes are 521 warps for the GPU's
+// 608 sub-partitions, and 645 by rows.  Address arithmetic is small beside the collision,
+// so nodes at the walls need no launch of their own (a ring launch on a second stream took
+// the step of a 64^2 cavity from 7 to 10 us with its fork and join).
+// GB300, us per step, the collision in FP64 with the ring apart / this: 64^2 13.1 / 7.2, 256^2
+// 39.2 / 14.4, 1024^2 505 / 154, 2048^2 1992 / 581; in place 1024^2 505 / 161; 101^2 with wall
+// nodes 23.6 / 16.  Bound by latency and issue (3,100 instructions per node, 49 % issue; FP64
+// pipe 53 % busy, against 83 % before).  4 blocks of 128 threads per SM (128 registers, 120
+// bytes of spills); 3 blocks (152 registers): 1024^2 165, 2048^2 633; 5 (96): 160, 603.
+constexpr int FLAT_MIN_BLOCKS = 4;
+
+template <bool EXT>
+__global__ void __launch_bounds__(128, FLAT_MIN_BLOCKS)
+step_ab_flat_kernel(const double* __restrict__ src, double* __restrict__ dst, double* __restrict__ hist, Geom G,
+                    Coef<double> c) {
+    pdl_trigger();
+    pdl_wait();                                // launched by launch_pdl()
+    const unsigned k = blockIdx.x * 128u + threadIdx.x;
+    if (k >= (unsigned)G.nx * (unsigned)G.ny) return;
+    const unsigned j = k / (unsigned)G.nx;
+    ab_node<double, EXT, false>(src, dst, hist, G, c, (int)(k - j * (unsigned)G.nx), (int)j);
+}
+
+// With nodes on the walls: the first blocks take the ring (its rebuild makes it the longest
+// chain), the others the inner nodes.
+template <bool EXT>
+__global__ void __launch_bounds__(128, FLAT_MIN_BLOCKS)
+step_ab_nee_flat_kernel(const double* __restrict__ src, double* __restrict__ dst, double* __restrict__ hist,
+                        Geom G, Coef<double> c, unsigned ring_blocks) {
+    pdl_trigger();
+    pdl_wait();                                // launched by launch_pdl()
+    int i, j;
+    double f[9], g[5], h[5], hv[4];
+    if (blockIdx.x < ring_blocks) {
+        const long long k = (long long)blockIdx.x * 128 + threadIdx.x;
+        if (k >= ring_count(G)) return;
+        ring_node(G, k, i, j);
+        gather_nee(src, G, i, j, c, f, g, h);
+    } else {
+        const unsigned k = (blockIdx.x - ring_blocks) * 128u + threadIdx.x, w = (unsigned)G.nx - 2u;
+        if (k >= w * ((unsigned)G.ny - 2u)) return;
+        j = (int)(k / w);
+        i = (int)(k - (unsigned)j * w) + 1;
+        j += 1;
+        gather_pull_inner<false, true>(src, G, (size_t)j * G.pitch + i, f, g, h);
+    }
+    // the collision's code once for both: the instruction cache holds it
+    const size_t self = (size_t)j * G.pitch + i;
+    load_hist(hist, G, self, hv);
+    uint32_t seed = 0;
+    collide_node<EXT>(c, self, G.plane, f, g, h, hv);
+    store_ab(dst, G, self, c, f, g, h, seed);
+    store_hist(hist, G, self, hv);
+}
+
+template <bool ODD, bool EXT>
+__global__ void __launch_bounds__(128, FLAT_MIN_BLOCKS)
+step_aa_flat_kernel(double* __restrict__ buf, double* __restrict__ hist, Geom G, Coef<double> c) {
+    pdl_trigger();
+    pdl_wait();                                // launched by launch_pdl()
+    const unsigned k = blockIdx.x * 128u + threadIdx.x;
+    if (k >= (unsigned)G.nx * (unsigned)G.ny) return;
+    const unsigned j = k / (unsigned)G.nx;
+    aa_node<double, ODD, EXT>(buf, hist, G, c, (int)(k - j * (unsigned)G.nx), (int)j);
+}
+
 // History (T u, C u) at t = 0 of the wall nodes, from their rebuilt initial state
 // (init_kernel wrote the interior's and the buffer the pull reads).
 template <typename S>
@@ -526,40 +652,6 @@ __global__ void nee_hist_kernel(const S* __restrict__ buf, typename Real<S>::typ
     const Macro<R> M = macro(cl, f, g, h);
     const R T = c.T0 + M.Tp, C = c.C0 + M.Cp;
     const R hv[4] = {T * M.ux, T * M.uy, C * M.ux, C * M.uy};
-    store_hist(hist, G, self, hv);
-}
-
-// ---- the fused step, in-place AA layout -------------------------------------------
-// Even step (level t even): natural pre-collision values at x -> collide ->
-// post-collision value of direction q stored in slot opp(q) of x.
-// Odd step: pull from the swapped slots of the neighbours (with wall rules),
-// collide, push post-collision value of direction q into slot q of x + e_q
-// (or, where that link crosses a wall, the reflected value into slot opp(q)
-// of x).  Each thread reads and writes the same set of locations, so the
-// update is race-free in place.
-template <typename S, bool ODD, bool EXT>
-__global__ void __launch_bounds__(256)
-step_aa_kernel(S* __restrict__ buf, typename Real<S>::type* __restrict__ hist, Geom G,
-               Coef<typename Real<S>::type> c) {
-    using R = typename Real<S>::type;
-    pdl_trigger();
-    pdl_wait();                                // launched by launch_pdl()
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    if (i >= G.nx || j >= G.ny) return;
-    R f[9], g[5], h[5], hv[4];
-    const size_t self = (size_t)j * G.pitch + i;
-    if (ODD)
-        gather_pull<true, true, EXT>(buf, G, i, j, c, f, g, h);
-    else
-        gather_local<true>(buf, G, i, j, f, g, h);
-    load_hist(hist, G, self, hv);
-    uint32_t seed = Store<S>::kLow ? node_seed(self, f[0], g[0]) : 0u;
-    collide_node<EXT>(c, self, G.plane, f, g, h, hv);
-    if (ODD)
-        store_aa_odd<EXT>(buf, G, i, j, self, c, f, g, h, seed);
-    else
-        store_aa_even(buf, G, self, c, f, g, h, seed);
     store_hist(hist, G, self, hv);
 }
 
@@ -614,7 +706,6 @@ __device__ __forceinline__ void aa_odd_ring_node(S* __restrict__ buf, R* __restr
     store_aa_odd<EXT>(buf, G, i, j, self, c, f, g, h, seed);
     store_hist(hist, G, self, hv);
 }
-__host__ __device__ inline long long ring_count(const Geom& G) { return 2LL * G.nx + 2LL * (G.ny - 2); }
 
 template <typename S, bool EXT>
 __global__ void __launch_bounds__(256)

@@ -57,16 +57,13 @@ inline bool pair_grid_aa_even(const Geom& G, dim3& gr) {
 // steps, one kernel / split with the ring on a second stream / split in one launch (the
 // ring's block rows first): 128^2 2.5 / 4.6 / 3.9, 256^2 2.9 / 4.9 / 4.6, 512^2 6.9 / 7.8 /
 // 6.3, 1024^2 28.2 / 27.5 / 25.5, 2048^2 121.3 / 117.0 / 114.6, 4096^2 - / 460.5 / 458.8.
-// FP64 splits at every size, the ring on a second stream (128^2 33.1 / 13.5 us, 1024^2
-// 507.5 / 502.3).
 #ifndef LBM_AA_SPLIT_MIN_NODES
 #define LBM_AA_SPLIT_MIN_NODES (1LL << 17)
 #endif
 // With FP32 arithmetic the split odd step is one launch (step_aa_odd_fused_kernel: the
 // ring's block rows, then the inner nodes), and so is the two-buffer step with wall nodes
 // (Sec. 3.3; step_ab_nee_fused_kernel): no second stream, no fork / join, a programmatic
-// dependent launch.  FP64 keeps the ring on a second stream beside the inner launch.  With
-// wall nodes, FP32, us per step (second stream / one launch): 1024^2 33.3 / 30.5, 4096^2
+// dependent launch.  With wall nodes, FP32, us per step (second stream / one launch): 1024^2 33.3 / 30.5, 4096^2
 // 459.2 / 456.7.
 #ifndef LBM_AA_ODD_FUSED
 #define LBM_AA_ODD_FUSED 1
@@ -99,7 +96,23 @@ cudaError_t launch_step_ab(const void* src, void* dst, void* hist, const Geom& G
             return launch_pdl(step_ab_pair_kernel<S>, gp, dim3(PAIR_BX, PAIR_BY), L.stream, (const S*)src,
                               (S*)dst, (float*)hist, G, c, erows);
     }
-    if constexpr (std::is_same<R, float>::value && LBM_AB_NEE_FUSED) {
+    if constexpr (std::is_same<S, double>::value) {
+        // one launch for all nodes, the wall nodes of Sec. 3.3 in its first blocks
+        const bool ext = c.poro || c.moving;
+        auto go = [&](auto* k, long long blocks, auto... more) {
+            return launch_pdl(k, dim3((unsigned)blocks), dim3(128), L.stream, (const S*)src, (S*)dst, (R*)hist, G, c,
+                              more...);
+        };
+        if (c.nee) {
+            const long long rb = (ring_count(G) + 127) / 128;
+            const long long ib = ((long long)(G.nx - 2) * (G.ny - 2) + 127) / 128;
+            return c.poro ? go(step_ab_nee_flat_kernel<true>, rb + ib, (unsigned)rb)
+                          : go(step_ab_nee_flat_kernel<false>, rb + ib, (unsigned)rb);
+        }
+        const long long nb = ((long long)G.nx * G.ny + 127) / 128;
+        return ext ? go(step_ab_flat_kernel<true>, nb) : go(step_ab_flat_kernel<false>, nb);
+    } else {
+    if constexpr (LBM_AB_NEE_FUSED) {
         if (c.nee) {
             // the ring of wall nodes (the rebuild, Sec. 3.3) in the first block rows, the
             // inner nodes (the plain pull) after them: one programmatic dependent launch
@@ -132,8 +145,8 @@ cudaError_t launch_step_ab(const void* src, void* dst, void* hist, const Geom& G
         return ring_join(L);
     } else if (!std::is_same<S, float>::value && G.nx >= 3 && G.ny >= 3) {
         // inner nodes with no wall logic, then the ring of outermost nodes.  GB300, 4096^2:
-        // BF16 385 -> 377 us, FP16 442 -> 410 us, FP64 (2048^2) 2201 -> 2148 us; the
-        // DRAM-bound FP32 step measured slower split (446 -> 460 us) and stays one kernel.
+        // BF16 385 -> 377 us, FP16 442 -> 410 us; the DRAM-bound FP32 step measured slower
+        // split (446 -> 460 us) and stays one kernel.
         const bool ext = c.poro || c.moving;
         cudaStream_t rs;
         cudaError_t e = ring_fork(L, &rs);
@@ -157,6 +170,7 @@ cudaError_t launch_step_ab(const void* src, void* dst, void* hist, const Geom& G
     if (c.poro || c.moving)
         return launch_pdl(step_ab_kernel<S, true>, gr, b, L.stream, (const S*)src, (S*)dst, (R*)hist, G, c);
     return launch_pdl(step_ab_kernel<S, false>, gr, b, L.stream, (const S*)src, (S*)dst, (R*)hist, G, c);
+    }
 }
 
 
@@ -178,8 +192,16 @@ cudaError_t launch_step_aa(void* buf, void* hist, const Geom& G,
                               c, erows);
         }
     }
-    const long long split_min = std::is_same<R, double>::value ? 0 : LBM_AA_SPLIT_MIN_NODES;
-    if constexpr (std::is_same<R, float>::value && LBM_AA_ODD_FUSED) {
+    if constexpr (std::is_same<S, double>::value) {
+        const long long nb = ((long long)G.nx * G.ny + 127) / 128;
+        auto go = [&](auto* k) {
+            return launch_pdl(k, dim3((unsigned)nb), dim3(128), L.stream, (S*)buf, (R*)hist, G, c);
+        };
+        if (odd) return ext ? go(step_aa_flat_kernel<true, true>) : go(step_aa_flat_kernel<true, false>);
+        return ext ? go(step_aa_flat_kernel<false, true>) : go(step_aa_flat_kernel<false, false>);
+    } else {
+    const long long split_min = LBM_AA_SPLIT_MIN_NODES;
+    if constexpr (LBM_AA_ODD_FUSED) {
         if (odd && G.nx >= 3 && G.ny >= 3 && (long long)G.nx * G.ny >= split_min) {
             // ring and inner nodes in one programmatic dependent launch (the ring's block
             // rows first)
@@ -220,6 +242,7 @@ cudaError_t launch_step_aa(void* buf, void* hist, const Geom& G,
     if (odd) return launch_pdl(step_aa_kernel<S, true, false>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
     if (ext) return launch_pdl(step_aa_kernel<S, false, true>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
     return launch_pdl(step_aa_kernel<S, false, false>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
+    }
 }
 
 template <typename S>
