@@ -7,6 +7,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -230,8 +231,48 @@ const char* check_params(const lbm_params& P) {
 
 }  // namespace
 
+// Pinned host memory that kernels write a context's few read-out numbers to (32 doubles a
+// context), so that a read-out waits for its kernel and for no copy behind it: a copy of
+// 32 bytes to pageable memory took 8 of the 29 us of a call.  One block of the process
+// serves up to 256 contexts; it is taken with the first and given back with the last.
+// A context without a slot copies its results as before.
+struct HostSlots {
+    static constexpr int kSlots = 256, kDoubles = 32;
+    std::mutex mu;
+    double* block = nullptr;
+    int used = 0;
+    bool taken[kSlots] = {};
+    double* take() {
+        std::lock_guard<std::mutex> lk(mu);
+        if (!block && cudaHostAlloc((void**)&block, sizeof(double) * kSlots * kDoubles,
+                                    cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            cudaGetLastError();
+            block = nullptr;
+            return nullptr;
+        }
+        for (int k = 0; k < kSlots; ++k)
+            if (!taken[k]) {
+                taken[k] = true;
+                ++used;
+                return block + (size_t)k * kDoubles;
+            }
+        return nullptr;
+    }
+    void give(double* p) {
+        if (!p) return;
+        std::lock_guard<std::mutex> lk(mu);
+        taken[(p - block) / kDoubles] = false;
+        if (--used == 0) {
+            cudaFreeHost(block);
+            block = nullptr;
+        }
+    }
+};
+HostSlots g_host_slots;
+
 // d_out: Nu/Sh of the side walls at 0, residual maxima at 8, Nu/Sh of bottom and top at
 // 20, scratch of the Nu/Sh pass at 64.
+constexpr int SMALL_CHUNK = 8;      // steps of the smaller captured chunk (even)
 constexpr int OUT_SCRATCH = 64, OUT_DOUBLES = OUT_SCRATCH + NUSH_SCRATCH;
 
 struct lbm_ctx {
@@ -244,6 +285,7 @@ struct lbm_ctx {
     void* hist_alt = nullptr;       // second history buffer (two steps per launch), or NULL
     int hcur = 0;                   // swaps of hist and hist_alt so far, mod 2
     double* d_out = nullptr;        // OUT_DOUBLES: Nu/Sh and residual results, Nu/Sh partial sums
+    double* h_out = nullptr;        // HostSlots::kDoubles of pinned memory laid out as d_out, or NULL
     double* d_fields = nullptr;     // lazily allocated [5][h][w] read-out window
     size_t fields_cap = 0;          // nodes d_fields holds
     void* d_snap = nullptr;         // lazily allocated [4][ny][nx] in the compute precision
@@ -265,9 +307,11 @@ struct lbm_ctx {
     LaunchCfg L{};
     int graph_chunk = 0;
     bool round_nearest = false;     // 16-bit storage: nearest-even instead of stochastic
-    // captured chunks by the buffers they start from: [2 * cur + hcur]
-    cudaGraphExec_t graph[4] = {nullptr, nullptr, nullptr, nullptr};
-    int graph_end[4] = {0, 0, 0, 0};   // and the buffers they end on
+    // captured chunks of graph_chunk steps and of a few (small_chunk), by the buffers they start
+    // from: [2 * cur + hcur], and the buffers they end on
+    cudaGraphExec_t graph[2][4] = {};
+    int graph_end[2][4] = {};
+    int64_t launched = 0;           // steps taken by launches of their own
     lbm_alloc_fn alloc = nullptr;
     lbm_free_fn free_fn = nullptr;
     void* alloc_user = nullptr;
@@ -367,6 +411,7 @@ cudaError_t two_steps(lbm_ctx* c) {
 cudaError_t enqueue(lbm_ctx* c, int64_t n) {
     cudaError_t e = cudaSuccess;
     const bool march = can_march(c);
+    c->launched += n;
     while (n > 0 && e == cudaSuccess) {
         if (march && n >= 2) {
             e = two_steps(c);
@@ -391,6 +436,17 @@ cudaError_t run_init(lbm_ctx* c, const InitSpec& I) {
 }
 
 const void* cur_buf(const lbm_ctx* c) { return c->layout == LBM_AB_PULL ? c->buf[c->cur] : c->buf[0]; }
+
+// Where the results at d_out + at go: the pinned slot, or device memory to copy from.
+inline double* out_at(const lbm_ctx* c, int at) { return (c->h_out ? c->h_out : c->d_out) + at; }
+// Fetches n of them after their kernel; waits for the stream.
+cudaError_t fetch(lbm_ctx* c, cudaError_t e, int at, int n, double* to) {
+    if (e == cudaSuccess && !c->h_out)
+        e = cudaMemcpyAsync(to, c->d_out + at, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e == cudaSuccess && c->h_out) std::memcpy(to, c->h_out + at, n * sizeof(double));
+    return e;
+}
 
 // (Re)initialise the state at t = 0 from host T / C fields or from the noise.
 lbm_status do_init(lbm_ctx* c, const double* T_host, const double* C_host, uint64_t seed,
@@ -442,6 +498,7 @@ bool lbm_ctx_view(const lbm_ctx* c, CtxView* v) {
     v->mode = c->read_mode();
     v->stream = c->stream;
     v->device = c->device;
+    v->host_out = c->h_out ? c->h_out + 8 : nullptr;
     return true;
 }
 
@@ -780,6 +837,7 @@ lbm_status create_core(const lbm_params* params, const lbm_options* opt, int sla
             c->hist_alt = c->dalloc(c->hist_bytes());
     }
     c->d_out = (double*)c->dalloc(OUT_DOUBLES * sizeof(double));
+    c->h_out = g_host_slots.take();
     if (O.eps_field || O.K_field) {
         if (c->P.model_a) {
             lbm_status s = c->fail(LBM_ERR_INVALID, "lbm_create: porous fields are not supported with model_a");
@@ -910,21 +968,28 @@ lbm_status lbm_step(lbm_ctx* c, int64_t n) {
         e = one_step(c);
         --n;
     }
-    if (c->graph_chunk > 0 && n >= c->graph_chunk && e == cudaSuccess) {
-        while (n >= c->graph_chunk && e == cudaSuccess) {
+    // chunks of graph_chunk steps; and, in a loop that takes a few steps at a time, of
+    // SMALL_CHUNK: a replay of those costs the host 6 us, their launches 33 (a capture, about
+    // 150 us, once a context has made 64 launches of its own)
+    for (int kind = 0; kind < 2 && c->graph_chunk > 0; ++kind) {
+        const int chunk = kind == 0 ? c->graph_chunk : SMALL_CHUNK;
+        if (kind == 1 && (c->launched < 64 || chunk >= c->graph_chunk)) break;
+        while (n >= chunk && e == cudaSuccess) {
             // a chunk is captured once per pair of buffers it can start from, and may end
             // on the others
             const int k0 = 2 * c->cur + c->hcur;
-            const int64_t t0 = c->t;
-            if (!c->graph[k0]) {
+            cudaGraphExec_t& graph = c->graph[kind][k0];
+            if (!graph) {
+                const int64_t t0 = c->t, launched0 = c->launched;
                 const int cur0 = c->cur, hcur0 = c->hcur;
                 void *h0 = c->hist, *h1 = c->hist_alt;
                 cudaGraph_t g = nullptr;
                 e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
                 if (e == cudaSuccess) {
-                    const cudaError_t le = enqueue(c, c->graph_chunk);
+                    const cudaError_t le = enqueue(c, chunk);
+                    c->graph_end[kind][k0] = 2 * c->cur + c->hcur;
                     c->t = t0;   // capture records, it does not run
-                    c->graph_end[k0] = 2 * c->cur + c->hcur;
+                    c->launched = launched0;
                     c->cur = cur0;
                     c->hcur = hcur0;
                     c->hist = h0;
@@ -932,23 +997,23 @@ lbm_status lbm_step(lbm_ctx* c, int64_t n) {
                     e = cudaStreamEndCapture(c->stream, &g);
                     if (le != cudaSuccess) e = le;
                 }
-                if (e == cudaSuccess) e = cudaGraphInstantiate(&c->graph[k0], g, 0);
+                if (e == cudaSuccess) e = cudaGraphInstantiate(&graph, g, 0);
                 if (g) cudaGraphDestroy(g);
                 if (e != cudaSuccess) {
-                    c->graph[k0] = nullptr;
+                    graph = nullptr;
                     return c->cuda_fail(e, "lbm_step: graph capture");
                 }
             }
-            e = cudaGraphLaunch(c->graph[k0], c->stream);
+            e = cudaGraphLaunch(graph, c->stream);
             if (e == cudaSuccess) {
-                const int k1 = c->graph_end[k0];
+                const int k1 = c->graph_end[kind][k0];
                 c->cur = k1 >> 1;
                 if ((k1 & 1) != c->hcur) {
                     std::swap(c->hist, c->hist_alt);
                     c->hcur ^= 1;
                 }
-                c->t += c->graph_chunk;
-                n -= c->graph_chunk;
+                c->t += chunk;
+                n -= chunk;
             }
         }
     }
@@ -1033,13 +1098,11 @@ lbm_status lbm_nusselt_sherwood(lbm_ctx* c, double out[4]) {
     W.L = c->P.nee ? c->P.nx - 1.0 : (double)c->P.nx;
     const int mode = c->read_mode();
     const void* b = cur_buf(c);
-    cudaError_t e = LBM_DISPATCH(c, launch_nush<double>(b, c->G, c->cd, mode, W, c->d_out + OUT_SCRATCH, c->d_out, c->stream),
-                                 launch_nush<float>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, c->d_out, c->stream),
-                                 launch_nush<__nv_bfloat16>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, c->d_out, c->stream),
-                                 launch_nush<__half>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, c->d_out, c->stream));
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(out, c->d_out, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    cudaError_t e = LBM_DISPATCH(c, launch_nush<double>(b, c->G, c->cd, mode, W, c->d_out + OUT_SCRATCH, out_at(c, 0), c->stream),
+                                 launch_nush<float>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, out_at(c, 0), c->stream),
+                                 launch_nush<__nv_bfloat16>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, out_at(c, 0), c->stream),
+                                 launch_nush<__half>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, out_at(c, 0), c->stream));
+    e = fetch(c, e, 0, 4, out);
     if (e != cudaSuccess) return c->cuda_fail(e, "lbm_nusselt_sherwood");
     for (int k = 0; k < 4; ++k)
         if (!std::isfinite(out[k]))
@@ -1068,13 +1131,11 @@ lbm_status lbm_nusselt_sherwood_tb(lbm_ctx* c, double out[4]) {
     W.L = c->P.nee ? c->P.ny - 1.0 : (double)c->P.ny;
     const int mode = c->read_mode();
     const void* b = cur_buf(c);
-    cudaError_t e = LBM_DISPATCH(c, launch_nush_tb<double>(b, c->G, c->cd, mode, W, c->d_out + OUT_SCRATCH, c->d_out + 20, c->stream),
-                                 launch_nush_tb<float>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, c->d_out + 20, c->stream),
-                                 launch_nush_tb<__nv_bfloat16>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, c->d_out + 20, c->stream),
-                                 launch_nush_tb<__half>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, c->d_out + 20, c->stream));
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(out, c->d_out + 20, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    cudaError_t e = LBM_DISPATCH(c, launch_nush_tb<double>(b, c->G, c->cd, mode, W, c->d_out + OUT_SCRATCH, out_at(c, 20), c->stream),
+                                 launch_nush_tb<float>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, out_at(c, 20), c->stream),
+                                 launch_nush_tb<__nv_bfloat16>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, out_at(c, 20), c->stream),
+                                 launch_nush_tb<__half>(b, c->G, c->cf, mode, W, c->d_out + OUT_SCRATCH, out_at(c, 20), c->stream));
+    e = fetch(c, e, 20, 4, out);
     if (e != cudaSuccess) return c->cuda_fail(e, "lbm_nusselt_sherwood_tb");
     for (int k = 0; k < 4; ++k)
         if (!std::isfinite(out[k]))
@@ -1094,18 +1155,19 @@ lbm_status residual_maxima(lbm_ctx* c, const char* who, double h[9]) {
         c->d_snap = c->dalloc(4 * n * c->rsz);
         c->d_partial = (double*)c->dalloc(RES_SCRATCH * sizeof(double));
         if (!c->d_snap || !c->d_partial) return c->fail(LBM_ERR_NOMEM, "%s: no device memory", who);
+        // every pass leaves its slots cleared for the next
+        const cudaError_t e = cudaMemsetAsync(c->d_partial, 0, RES_SCRATCH * sizeof(double), c->stream);
+        if (e != cudaSuccess) return c->cuda_fail(e, who);
     }
     const int mode = c->read_mode();
     const void* b = cur_buf(c);
-    double* o = c->d_out + 8;
+    double* o = out_at(c, 8);
     cudaError_t e = LBM_DISPATCH(
         c, launch_residual<double>(b, c->G, c->cd, mode, c->d_snap, c->d_partial, o, c->stream),
         launch_residual<float>(b, c->G, c->cf, mode, c->d_snap, c->d_partial, o, c->stream),
         launch_residual<__nv_bfloat16>(b, c->G, c->cf, mode, c->d_snap, c->d_partial, o, c->stream),
         launch_residual<__half>(b, c->G, c->cf, mode, c->d_snap, c->d_partial, o, c->stream));
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(h, o, 9 * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    e = fetch(c, e, 8, 9, h);
     if (e != cudaSuccess) return c->cuda_fail(e, who);
     if (h[8] != 0.0) return c->fail(LBM_ERR_DIVERGED, "%s: non-finite field at t=%lld", who, (long long)c->t);
     if (!c->snap_valid)   // no earlier fields: the changes are unknown
@@ -1335,10 +1397,11 @@ lbm_status lbm_load(lbm_ctx* c, const void* buf, size_t len) {
     c->cf.seed_off = (long long)(c->slab_y0 - c->G.jb) * c->G.pitch;
     c->cd.poro = (c->poro && c->rsz == 8) ? (const double*)c->poro : nullptr;
     c->cf.poro = (c->poro && c->rsz == 4) ? (const float*)c->poro : nullptr;
-    for (cudaGraphExec_t& g : c->graph) {   // constants are baked into the captured launches
-        if (g) cudaGraphExecDestroy(g);
-        g = nullptr;
-    }
+    for (auto& kind : c->graph)             // constants are baked into the captured launches
+        for (cudaGraphExec_t& g : kind) {
+            if (g) cudaGraphExecDestroy(g);
+            g = nullptr;
+        }
     c->t = h.t;
     c->cur = slot;
     c->snap_valid = false;
@@ -1360,13 +1423,15 @@ void lbm_destroy(lbm_ctx* c) {
     if (!c) return;
     DeviceGuard dg(c->device);
     if (c->stream) cudaStreamSynchronize(c->stream);
-    for (cudaGraphExec_t g : c->graph)
-        if (g) cudaGraphExecDestroy(g);
+    for (auto& kind : c->graph)
+        for (cudaGraphExec_t g : kind)
+            if (g) cudaGraphExecDestroy(g);
     c->dfree(c->buf[0], c->state_bytes());
     c->dfree(c->buf[1], c->state_bytes());
     c->dfree(c->hist, c->hist_bytes());
     c->dfree(c->hist_alt, c->hist_bytes());
     c->dfree(c->d_out, OUT_DOUBLES * sizeof(double));
+    g_host_slots.give(c->h_out);
     c->dfree(c->d_fields, 5 * c->fields_cap * sizeof(double));
     c->dfree(c->d_snap, 4 * c->nodes() * c->rsz);
     c->dfree(c->d_partial, RES_SCRATCH * sizeof(double));

@@ -1018,7 +1018,7 @@ nush_kernel(const S* __restrict__ buf, Geom G, Coef<typename Real<S>::type> c, i
 // atomicMax on the FP64 bit patterns (all values are >= 0, whose bit patterns
 // order as the values do); the block that finishes last folds the slots into out[9].
 // Slots and the block count behind them (slots[RES_SLOTS * 9]) must be zero before the
-// launch.  Block (bx, by) takes the 256-column tiles bx, bx + gridDim.x, ... of the rows
+// launch, and are again after it.  Block (bx, by) takes the 256-column tiles bx, bx + gridDim.x, ... of the rows
 // by, by + gridDim.y, ...; with the grid of residual_grid() that is one node per thread.
 // Maxima of FP64 values go through their bit patterns too: the FP64 pipe is the
 // scarce one.  A launch of its own that folded 4096 slots with FP64 maxima took 24 us;
@@ -1135,16 +1135,16 @@ residual_kernel(const S* __restrict__ buf, Geom G, Coef<typename Real<S>::type> 
             m = max_bits(m, *(volatile unsigned long long*)(slots + (size_t)b * 9 + q));
         m = warp_max_bits(m);
         if (lane == 0) out[q] = __longlong_as_double((long long)m);
+        for (int b = lane; b < RES_SLOTS; b += 32) slots[(size_t)b * 9 + q] = 0;   // for the next pass
     }
+    if (threadIdx.x == 0) slots[RES_SLOTS * 9] = 0;
 }
 
-// Clears the slots and launches the pass with the gather mode and the porous-field
+// Launches the pass with the gather mode and the porous-field
 // code fixed at compile time.
 template <typename S, typename P>
 cudaError_t launch_residual_pass(const S* buf, const Geom& G, const Coef<typename Real<S>::type>& c,
                                  int mode, P* snap, double* slots, double* out, cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(slots, 0, RES_SCRATCH * sizeof(double), st);
-    if (e != cudaSuccess) return e;
     const dim3 grid = residual_grid(G);
     unsigned long long* sl = reinterpret_cast<unsigned long long*>(slots);
 #define LBM_RES_CASE(M)                                                                          \

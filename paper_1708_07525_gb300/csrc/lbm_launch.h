@@ -111,7 +111,8 @@ template <typename S>
 cudaError_t launch_nush_tb(const void* buf, const Geom& G, const Coef<typename Real<S>::type>& c,
                            int mode, const WallSpec& W, double* scratch, double* out, cudaStream_t st);
 // snap holds 4 * nx * ny values of the compute precision (FP64 for FP64 storage,
-// else FP32); partial must hold RES_SCRATCH doubles; out 9 doubles.
+// else FP32); partial must hold RES_SCRATCH doubles, zero at the first call and left zero by
+// each; out 9 doubles.
 template <typename S>
 cudaError_t launch_residual(const void* buf, const Geom& G, const Coef<typename Real<S>::type>& c,
                             int mode, void* snap, double* partial, double* out,
@@ -166,6 +167,7 @@ struct CtxView {
     int mode;                // GATHER_* for the current level
     cudaStream_t stream;
     int device;
+    double* host_out;        // nine doubles of pinned memory for the residual's maxima, or NULL
 };
 
 }  // namespace lbm

@@ -11,6 +11,7 @@
 
 #include <cmath>
 #include <cstdio>
+#include <cstring>
 #include <mutex>
 
 #include "../../include/lbm.h"
@@ -58,8 +59,11 @@ template <typename S>
 cudaError_t launch(const CtxView& v, double* snap, double* scratch) {
     using R = typename Real<S>::type;
     const Coef<R>& c = coef_of(v, (R*)nullptr);
+    // the shared array may hold what a call that raced with another one left
+    cudaError_t e = cudaMemsetAsync(scratch, 0, RES_SCRATCH * sizeof(double), v.stream);
+    if (e != cudaSuccess) return e;
     return launch_residual_pass<S, double>((const S*)v.buf, v.G, c, v.mode, snap, scratch,
-                                           scratch + NOALLOC_OUT, v.stream);
+                                           v.host_out ? v.host_out : scratch + NOALLOC_OUT, v.stream);
 }
 
 lbm_status fail(lbm_ctx* ctx, lbm_status s, const char* m, const char* detail = "") {
@@ -94,9 +98,10 @@ lbm_status lbm_residual_noalloc(lbm_ctx* ctx, double* snapshot, int have_snapsho
         default: e = launch<__half>(v, snapshot, scratch); break;
     }
     double h[9];
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && !v.host_out)
         e = cudaMemcpyAsync(h, scratch + NOALLOC_OUT, sizeof h, cudaMemcpyDeviceToHost, v.stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(v.stream);
+    if (e == cudaSuccess && v.host_out) std::memcpy(h, v.host_out, sizeof h);
     if (e != cudaSuccess) return fail(ctx, LBM_ERR_CUDA, "", cudaGetErrorString(e));
     if (h[8] != 0.0) return fail(ctx, LBM_ERR_DIVERGED, "non-finite field value");
     double res = 0.0;

@@ -47,3 +47,36 @@ def test_wall_numbers_and_residual_match_the_fields(nx, ny, kind, precision):
     u = 2.0 ** -52 if precision == "f64" else 2.0 ** -23
     r = max(np.abs(now[k] - before[k]).max() / np.abs(now[k]).max() for k in ("ux", "uy", "T", "C"))
     np.testing.assert_allclose(c.residual(), r, rtol=0, atol=4 * u)
+
+
+@pytest.mark.parametrize("precision,layout,n", [("f32", "ab", 129), ("f32", "aa", 40), ("f64", "ab", 33),
+                                                ("f32", "ab", 900)])
+def test_a_few_steps_at_a_time(precision, layout, n):
+    """A loop of short step calls, which replays captured chunks of eight steps after 64
+    launches, takes the same steps as one call, from even and odd levels."""
+    kw = dict(precision=precision, layout=layout, seed=2, noise=0.02)
+    a = lbm.Cavity(n, n, 1e4, 1e-2, 0.6, 1.0, 2.0, 1.0, **kw)
+    b = lbm.Cavity(n, n, 1e4, 1e-2, 0.6, 1.0, 2.0, 1.0, graph_chunk=-1, **kw)
+    calls = [10, 9, 17, 8, 31, 1, 8, 16, 11, 24, 3, 40]
+    for _ in range(2):
+        for k in calls:
+            a.step(k)
+    b.step(2 * sum(calls))
+    fa, fb = a.fields(), b.fields()
+    for k in fa:
+        assert np.array_equal(fa[k], fb[k]), k
+
+
+def test_more_contexts_than_pinned_slots():
+    """256 contexts read out through pinned memory, the others through copies; slots are
+    taken again after contexts are gone."""
+    made = [lbm.Cavity(8, 6, 1e4, 1e-2, 0.6, 1.0, 2.0, 1.0, precision="f32", seed=k) for k in range(262)]
+    for c in made:
+        c.step(2)
+    got = [(tuple(c.nusselt_sherwood()), c.residual(), c.residual_parts()[4:].tolist()) for c in made]
+    for c in made[:100]:
+        c.close()
+    for k in (0, 3, 255, 256, 261):
+        c = lbm.Cavity(8, 6, 1e4, 1e-2, 0.6, 1.0, 2.0, 1.0, precision="f32", seed=k)
+        c.step(2)
+        assert (tuple(c.nusselt_sherwood()), c.residual(), c.residual_parts()[4:].tolist()) == got[k]
