@@ -36,7 +36,8 @@ KERNEL_SOURCES = ["paper_1708_07525_gb300/csrc/lbm_kernels.cuh",
                   "paper_1708_07525_gb300/csrc/lbm_device.cuh",
                   "paper_1708_07525_gb300/csrc/lbm_launchers.cuh",
                   "paper_1708_07525_gb300/csrc/lbm_march.cuh",
-                  "paper_1708_07525_gb300/csrc/lbm_fixed.cuh"]
+                  "paper_1708_07525_gb300/csrc/lbm_fixed.cuh",
+                  "paper_1708_07525_gb300/csrc/lbm_trio.cuh"]
 
 
 def kernel_hash() -> str:

@@ -87,91 +87,60 @@ __device__ __forceinline__ long long fx_shift(long long v, int d) {
 
 __device__ __forceinline__ int fx_max(int a, int b) { return a > b ? a : b; }
 
-// One D2Q5 lattice (collide_d2q5): d as integers of scale E, their sum s; (Px, Py) = Phi u now
-// and (Qx, Qy) before.  The populations leave in d.
-__device__ __forceinline__ void fixed_d2q5(double d[5], long long v[5], int E, long long s, double Px,
-                                                    double Py, double Qx, double Qy,
-                                                    const FixedScalar& r) {
-    // a scale that holds the fluxes as well (a bit of headroom above it)
-    const int need = fx_max(fx_max(fx_exp(Px), fx_exp(Py)), fx_max(fx_exp(Qx), fx_exp(Qy))) - 1;
-    if (need > E) {
-        for (int q = 0; q < 5; ++q) v[q] = fx_shift(v[q], need - E);
-        s = fx_shift(s, need - E);
-        E = need;
-    }
-    const long long px = fx_in(Px, E), py = fx_in(Py, E);
-    const long long p13 = v[1] + v[3], p24 = v[2] + v[4];
-    const long long b1 = fx_minus(v[1] - v[3] - px, r.b1, px - fx_in(Qx, E), r.q1, r.less1);
-    const long long b2 = fx_minus(v[2] - v[4] - py, r.b2, py - fx_in(Qy, E), r.q2, r.less2);
-    const long long b3 = fx_plus(p13 + p24 - 4 * v[0], r.b3, r.p_neg ? -s : s, r.p, r.less3);
-    const long long b4 = fx_one(p13 - p24, r.b4, r.less4);
-    const long long X = b3 + b4, Y = b3 - b4;
-    d[0] = fx_out(v[0] + 4 * b3, E);
-    d[1] = fx_out(v[1] - X - b1, E);
-    d[2] = fx_out(v[2] - Y - b2, E);
-    d[3] = fx_out(v[3] - X + b1, E);
-    d[4] = fx_out(v[4] - Y + b2, E);
-}
-
-// collide() of one FP64 node with uniform porous constants (the same update; see
-// collide_flow for the algebra).
-__device__ __forceinline__ void collide_fixed(const Coef<double>& c, double f[9], double g[5],
-                                                       double h[5], double hist[4]) {
-    const FixedCoef& k = c.fx;
-    int E = FX_LOW, Eg = FX_LOW, Eh = FX_LOW;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) E = fx_max(E, fx_exp(f[q]));
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-        Eg = fx_max(Eg, fx_exp(g[q]));
-        Eh = fx_max(Eh, fx_exp(h[q]));
-    }
-    long long v[9], vg[5], vh[5];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-        vg[q] = fx_in(g[q], Eg);
-        vh[q] = fx_in(h[q], Eh);
-    }
-    const long long sg = vg[0] + (vg[1] + vg[3]) + (vg[2] + vg[4]), sh = vh[0] + (vh[1] + vh[3]) + (vh[2] + vh[4]);
-#pragma unroll
-    for (int q = 0; q < 9; ++q) v[q] = fx_in(f[q], E);
-    long long d13 = v[1] - v[3], d24 = v[2] - v[4], D57 = v[5] - v[7], D68 = v[6] - v[8];
-    const double jx = fx_out(d13 + D57 - D68, E), jy = fx_out(d24 + D57 + D68, E);
-    // macro(): Eqs. 26, 6, 19, 18, 5
-    const double Tp = mul_(fx_out(sg, Eg), c.inv_sigma), Cp = mul_(fx_out(sh, Eh), c.inv_eps);
+// u, F of Eqs. 18, 5 (macro() from the moments).
+struct FixedMacro {
+    double ux, uy, Fx, Fy;
+};
+__device__ __forceinline__ FixedMacro fixed_macro(const Coef<double>& c, double jx, double jy, double Tp, double Cp) {
     const double Gy = fma_(c.gbT, Tp, mul_(c.gbC, Cp));
     const double vx = add_(jx, c.half_epsGx), vy = fma_(c.half_eps, Gy, jy);
     const double vm = sqrt_pos<false>(fma_(vx, vx, fma_(vy, vy, tiny_<double>())));
     const double inv_den = rcp_pos<false>(add_(c.l0, sqrt_pos<false>(fma_(c.l1, vm, c.l0sq))));
-    const double ux = mul_(vx, inv_den), uy = mul_(vy, inv_den);
+    FixedMacro M;
+    M.ux = mul_(vx, inv_den);
+    M.uy = mul_(vy, inv_den);
     const double ndrag = fma_(c.ndrag_quad, mul_(vm, inv_den), c.ndrag_lin);
-    const double Fx = fma_(ndrag, ux, c.epsGx), Fy = fma_(ndrag, uy, mul_(c.eps, Gy));
+    M.Fx = fma_(ndrag, M.ux, c.epsGx);
+    M.Fy = fma_(ndrag, M.uy, mul_(c.eps, Gy));
+    return M;
+}
+
+// The largest exponents of a lattice, at least FX_LOW, and its populations on that scale.
+template <int N> __device__ __forceinline__ int fixed_in(const double* d, long long* v) {
+    int E = FX_LOW;
+#pragma unroll
+    for (int q = 0; q < N; ++q) E = fx_max(E, fx_exp(d[q]));
+#pragma unroll
+    for (int q = 0; q < N; ++q) v[q] = fx_in(d[q], E);
+    return E;
+}
+template <int N> __device__ __forceinline__ void fixed_nan(double* d) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) d[q] = __longlong_as_double(0x7FF8000000000000ll);
+}
+constexpr int FX_TOP = 0x7FF - 8;        // exponents from here on count as not finite
+
+// The D2Q9 update (collide_flow): f as integers v of scale E; `top` the largest exponent of the
+// node so far.  The populations leave in f.
+__device__ __forceinline__ void fixed_flow(const Coef<double>& c, const FixedMacro& M, double f[9], long long v[9],
+                                           int E, int top) {
+    const FixedCoef& k = c.fx;
+    const double ux = M.ux, uy = M.uy, Fx = M.Fx, Fy = M.Fy;
     const double uxe = mul_(ux, c.inv_eps_f), uye = mul_(uy, c.inv_eps_f);
     const double dA = mul_(ux, uxe), dB = mul_(uy, uye), dXY = mul_(ux, uye);
     const double dP = mul_(uxe, Fx), dQ = mul_(uye, Fy), dW = fma_(uxe, Fy, mul_(uye, Fx));
-    const double T = add_(c.T0, Tp), C = add_(c.C0, Cp);
-    const double Tux = mul_(T, ux), Tuy = mul_(T, uy), Cux = mul_(C, ux), Cuy = mul_(C, uy);
-    // not finite somewhere: everything becomes NaN
-    int top = fx_max(fx_max(E, Eg), Eh);
-    const double all[] = {Tux, Tuy, Cux, Cuy, dA, dB, dP, dQ, dW, hist[0], hist[1], hist[2], hist[3]};
-#pragma unroll
-    for (int i = 0; i < 13; ++i) top = fx_max(top, fx_exp(all[i]));
-    if (top >= 0x7FF - 8) {
-        const double nan = __longlong_as_double(0x7FF8000000000000ll);
-#pragma unroll
-        for (int q = 0; q < 9; ++q) f[q] = nan;
-#pragma unroll
-        for (int q = 0; q < 5; ++q) g[q] = h[q] = nan;
+    // a scale that holds u, F and their products too (a bit of headroom above it)
+    const int most = fx_max(fx_max(fx_max(fx_exp(ux), fx_exp(uy)), fx_max(fx_exp(Fx), fx_exp(Fy))),
+                            fx_max(fx_max(fx_exp(dA), fx_exp(dB)), fx_max(fx_exp(dW), fx_max(fx_exp(dP), fx_exp(dQ)))));
+    if (fx_max(top, most) >= FX_TOP) {
+        fixed_nan<9>(f);
         return;
     }
-    // the flow lattice: a scale that holds u, F and their products too
-    const int need = fx_max(fx_max(fx_max(fx_exp(ux), fx_exp(uy)), fx_max(fx_exp(Fx), fx_exp(Fy))),
-                            fx_max(fx_max(fx_exp(dA), fx_exp(dB)), fx_max(fx_exp(dW), fx_max(fx_exp(dP), fx_exp(dQ))))) - 1;
-    if (need > E) {
-        for (int q = 0; q < 9; ++q) v[q] = fx_shift(v[q], need - E);
-        E = need;
-        d13 = v[1] - v[3], d24 = v[2] - v[4], D57 = v[5] - v[7], D68 = v[6] - v[8];
+    if (most - 1 > E) {
+        for (int q = 0; q < 9; ++q) v[q] = fx_shift(v[q], most - 1 - E);
+        E = most - 1;
     }
+    const long long d13 = v[1] - v[3], d24 = v[2] - v[4], D57 = v[5] - v[7], D68 = v[6] - v[8];
     const long long p13 = v[1] + v[3], p24 = v[2] + v[4], p57 = v[5] + v[7], p68 = v[6] + v[8];
     const long long fa = p13 + p24, fd = p57 + p68;
     const long long A = fx_in(dA, E), B = fx_in(dB, E), P = fx_in(dP, E), Q = fx_in(dQ, E);
@@ -196,12 +165,64 @@ __device__ __forceinline__ void collide_fixed(const Coef<double>& c, double f[9]
     f[6] = fx_out(v[6] - V - t, E);
     f[7] = fx_out(v[7] - U - r, E);
     f[8] = fx_out(v[8] + t - V, E);
-    fixed_d2q5(g, vg, Eg, sg, Tux, Tuy, hist[0], hist[1], k.zs);
-    fixed_d2q5(h, vh, Eh, sh, Cux, Cuy, hist[2], hist[3], k.es);
-    hist[0] = Tux;
-    hist[1] = Tuy;
-    hist[2] = Cux;
-    hist[3] = Cuy;
+}
+
+// One D2Q5 lattice (collide_d2q5): d as integers v of scale E, their sum s; Phi the scalar's value;
+// hist Phi u before, replaced by Phi u now.  The populations leave in d.
+__device__ __forceinline__ void fixed_scalar(const FixedScalar& r, double Phi, const FixedMacro& M, double d[5],
+                                             long long v[5], int E, long long s, double hist[2], int top) {
+    const double Px = mul_(Phi, M.ux), Py = mul_(Phi, M.uy), Qx = hist[0], Qy = hist[1];
+    hist[0] = Px;
+    hist[1] = Py;
+    // a scale that holds the fluxes as well (a bit of headroom above it)
+    const int most = fx_max(fx_max(fx_exp(Px), fx_exp(Py)), fx_max(fx_exp(Qx), fx_exp(Qy)));
+    if (fx_max(top, most) >= FX_TOP) {
+        fixed_nan<5>(d);
+        return;
+    }
+    if (most - 1 > E) {
+        for (int q = 0; q < 5; ++q) v[q] = fx_shift(v[q], most - 1 - E);
+        s = fx_shift(s, most - 1 - E);
+        E = most - 1;
+    }
+    const long long px = fx_in(Px, E), py = fx_in(Py, E);
+    const long long p13 = v[1] + v[3], p24 = v[2] + v[4];
+    const long long b1 = fx_minus(v[1] - v[3] - px, r.b1, px - fx_in(Qx, E), r.q1, r.less1);
+    const long long b2 = fx_minus(v[2] - v[4] - py, r.b2, py - fx_in(Qy, E), r.q2, r.less2);
+    const long long b3 = fx_plus(p13 + p24 - 4 * v[0], r.b3, r.p_neg ? -s : s, r.p, r.less3);
+    const long long b4 = fx_one(p13 - p24, r.b4, r.less4);
+    const long long X = b3 + b4, Y = b3 - b4;
+    d[0] = fx_out(v[0] + 4 * b3, E);
+    d[1] = fx_out(v[1] - X - b1, E);
+    d[2] = fx_out(v[2] - Y - b2, E);
+    d[3] = fx_out(v[3] - X + b1, E);
+    d[4] = fx_out(v[4] - Y + b2, E);
+}
+
+// The momentum and a scalar's sum from integers.
+__device__ __forceinline__ double fixed_jx(const long long v[9], int E) {
+    return fx_out(v[1] - v[3] + v[5] - v[7] - v[6] + v[8], E);
+}
+__device__ __forceinline__ double fixed_jy(const long long v[9], int E) {
+    return fx_out(v[2] - v[4] + v[5] - v[7] + v[6] - v[8], E);
+}
+__device__ __forceinline__ long long fixed_sum(const long long v[5]) {
+    return v[0] + (v[1] + v[3]) + (v[2] + v[4]);
+}
+
+// collide() of one FP64 node with uniform porous constants (the same update; see
+// collide_flow for the algebra).
+__device__ __forceinline__ void collide_fixed(const Coef<double>& c, double f[9], double g[5], double h[5],
+                                              double hist[4]) {
+    long long v[9], vg[5], vh[5];
+    const int E = fixed_in<9>(f, v), Eg = fixed_in<5>(g, vg), Eh = fixed_in<5>(h, vh);
+    const long long sg = fixed_sum(vg), sh = fixed_sum(vh);
+    const double Tp = mul_(fx_out(sg, Eg), c.inv_sigma), Cp = mul_(fx_out(sh, Eh), c.inv_eps);     // Eq. 26
+    const FixedMacro M = fixed_macro(c, fixed_jx(v, E), fixed_jy(v, E), Tp, Cp);
+    const int top = fx_max(fx_max(E, Eg), Eh);
+    fixed_flow(c, M, f, v, E, top);
+    fixed_scalar(c.fx.zs, add_(c.T0, Tp), M, g, vg, Eg, sg, hist, top);
+    fixed_scalar(c.fx.es, add_(c.C0, Cp), M, h, vh, Eh, sh, hist + 2, top);
 }
 
 }  // namespace lbm

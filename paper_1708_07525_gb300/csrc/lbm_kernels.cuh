@@ -188,6 +188,52 @@ __device__ __forceinline__ R nee_scalar(const Coef<R>& c, int di, int dj, const 
     return fma_(fnma_(den, q, num), r, q);
 }
 
+// f of Eq. 33 on a wall node from x_f's: (ux, uy) there, (ubx, uby) the wall's, ief and ieb
+// 1 / eps of the two (0 without the nonlinear term).
+template <typename R>
+__device__ __forceinline__ void nee_flow(R ux, R uy, R ubx, R uby, R ief, R ieb, R f[9]) {
+    // Q(u_w) - Q(u_f) = 3 e . d + 4.5 e . A e - 1.5 tr A with d = u_w - u_f and the tensor
+    // A = u_w u_w / eps_b - u_f u_f / eps_f
+    const R fex = mul_(ux, ief), fey = mul_(uy, ief), bex = mul_(ubx, ieb), bey = mul_(uby, ieb);
+    const R Axx = fma_(ubx, bex, -mul_(ux, fex)), Ayy = fma_(uby, bey, -mul_(uy, fey));
+    const R Axy = mul_(R(0.25), fma_(ubx, bey, -mul_(ux, fey)));
+    const R tr = add_(Axx, Ayy), diag = mul_(R(1.0 / 12.0), tr);
+    const R dx = sub_(ubx, ux), dy = sub_(uby, uy);
+    const R axx = mul_(R(1.0 / 6.0), fma_(R(3), Axx, -tr)), axy = mul_(R(1.0 / 6.0), fma_(R(3), Ayy, -tr));
+    f[0] = fma_(R(-2.0 / 3.0), tr, f[0]);
+    f[1] = add_(f[1], fma_(R(1.0 / 3.0), dx, axx));
+    f[2] = add_(f[2], fma_(R(1.0 / 3.0), dy, axy));
+    f[3] = add_(f[3], fma_(R(-1.0 / 3.0), dx, axx));
+    f[4] = add_(f[4], fma_(R(-1.0 / 3.0), dy, axy));
+    const R dp = mul_(R(1.0 / 12.0), add_(dx, dy)), dm = mul_(R(1.0 / 12.0), sub_(dx, dy));
+    f[5] = add_(f[5], add_(add_(diag, Axy), dp));
+    f[6] = add_(f[6], sub_(sub_(diag, Axy), dm));
+    f[7] = add_(f[7], sub_(add_(diag, Axy), dp));
+    f[8] = add_(f[8], add_(sub_(diag, Axy), dm));
+}
+// The four moving populations of Eq. 34 / 35: a the equilibrium's change, j half the flux's.
+template <typename R>
+__device__ __forceinline__ void nee_moving(R a, R ux, R uy, R ubx, R uby, R F, R B, R d[5]) {
+    const R jx = mul_(R(0.5), fma_(ubx, B, -mul_(ux, F))), jy = mul_(R(0.5), fma_(uby, B, -mul_(uy, F)));
+    d[1] = add_(d[1], add_(a, jx));
+    d[2] = add_(d[2], add_(a, jy));
+    d[3] = add_(d[3], sub_(a, jx));
+    d[4] = add_(d[4], sub_(a, jy));
+}
+// g of Eq. 34 and h of Eq. 35, from the scalar's deviation at x_f and on the wall.
+template <typename R>
+__device__ __forceinline__ void nee_heat(const Coef<R>& c, R ux, R uy, R ubx, R uby, R Tf, R Tb, R g[5]) {
+    const R dT = sub_(Tb, Tf);
+    g[0] = fma_(c.aT0, dT, g[0]);
+    nee_moving(mul_(c.aT1, dT), ux, uy, ubx, uby, add_(c.T0, Tf), add_(c.T0, Tb), g);
+}
+template <typename R>
+__device__ __forceinline__ void nee_mass(const Coef<R>& c, const Coef<R>& cf, const Coef<R>& cb, R ux, R uy, R ubx,
+                                         R uby, R Cf, R Cb, R h[5]) {
+    h[0] = add_(h[0], fma_(cb.aC0, Cb, -mul_(cf.aC0, Cf)));
+    nee_moving(fma_(cb.aC1, Cb, -mul_(cf.aC1, Cf)), ux, uy, ubx, uby, add_(c.C0, Cf), add_(c.C0, Cb), h);
+}
+
 // Pre-collision populations (deviations) of wall node (i, j) with inward link (di, dj)
 // in the two-buffer pull layout, rebuilt by Eqs. 33-35 from the nearest interior node
 // x_f = (i + di, j + dj) and, for the wall value, x_ff = (i + 2 di, j + 2 dj):
@@ -219,40 +265,9 @@ __device__ __forceinline__ void nee_rebuild(const S* __restrict__ buf, const Geo
     const R Cb = nee_scalar(c, di, dj, c.CwP, c.bC, M.Cp, Cff);
     const int sv = dj ? (dj > 0 ? 2 : 3) : (di > 0 ? 0 : 1);
     const R ubx = c.uwall[sv][0], uby = c.uwall[sv][1];
-    // Q(u_w) - Q(u_f) = 3 e . d + 4.5 e . A e - 1.5 tr A with d = u_w - u_f and the tensor
-    // A = u_w u_w / eps_b - u_f u_f / eps_f
-    const R ieb = cb.inv_eps_f, ief = cf.inv_eps_f;
-    const R fex = mul_(M.ux, ief), fey = mul_(M.uy, ief), bex = mul_(ubx, ieb), bey = mul_(uby, ieb);
-    const R Axx = fma_(ubx, bex, -mul_(M.ux, fex)), Ayy = fma_(uby, bey, -mul_(M.uy, fey));
-    const R Axy = mul_(R(0.25), fma_(ubx, bey, -mul_(M.ux, fey)));
-    const R tr = add_(Axx, Ayy), diag = mul_(R(1.0 / 12.0), tr);
-    const R dx = sub_(ubx, M.ux), dy = sub_(uby, M.uy);
-    const R axx = mul_(R(1.0 / 6.0), fma_(R(3), Axx, -tr)), axy = mul_(R(1.0 / 6.0), fma_(R(3), Ayy, -tr));
-    f[0] = fma_(R(-2.0 / 3.0), tr, f[0]);
-    f[1] = add_(f[1], fma_(R(1.0 / 3.0), dx, axx));
-    f[2] = add_(f[2], fma_(R(1.0 / 3.0), dy, axy));
-    f[3] = add_(f[3], fma_(R(-1.0 / 3.0), dx, axx));
-    f[4] = add_(f[4], fma_(R(-1.0 / 3.0), dy, axy));
-    const R dp = mul_(R(1.0 / 12.0), add_(dx, dy)), dm = mul_(R(1.0 / 12.0), sub_(dx, dy));
-    f[5] = add_(f[5], add_(add_(diag, Axy), dp));
-    f[6] = add_(f[6], sub_(sub_(diag, Axy), dm));
-    f[7] = add_(f[7], sub_(add_(diag, Axy), dp));
-    f[8] = add_(f[8], add_(sub_(diag, Axy), dm));
-    const R TB = add_(c.T0, Tb), TF = add_(c.T0, M.Tp), CB = add_(c.C0, Cb), CF = add_(c.C0, M.Cp);
-    const R dT = sub_(Tb, M.Tp), gT = mul_(c.aT1, dT);
-    const R jTx = mul_(R(0.5), fma_(ubx, TB, -mul_(M.ux, TF))), jTy = mul_(R(0.5), fma_(uby, TB, -mul_(M.uy, TF)));
-    const R gC = fma_(cb.aC1, Cb, -mul_(cf.aC1, M.Cp));
-    const R jCx = mul_(R(0.5), fma_(ubx, CB, -mul_(M.ux, CF))), jCy = mul_(R(0.5), fma_(uby, CB, -mul_(M.uy, CF)));
-    g[0] = fma_(c.aT0, dT, g[0]);
-    h[0] = add_(h[0], fma_(cb.aC0, Cb, -mul_(cf.aC0, M.Cp)));
-    g[1] = add_(g[1], add_(gT, jTx));
-    g[2] = add_(g[2], add_(gT, jTy));
-    g[3] = add_(g[3], sub_(gT, jTx));
-    g[4] = add_(g[4], sub_(gT, jTy));
-    h[1] = add_(h[1], add_(gC, jCx));
-    h[2] = add_(h[2], add_(gC, jCy));
-    h[3] = add_(h[3], sub_(gC, jCx));
-    h[4] = add_(h[4], sub_(gC, jCy));
+    nee_flow(M.ux, M.uy, ubx, uby, cf.inv_eps_f, cb.inv_eps_f, f);
+    nee_heat(c, M.ux, M.uy, ubx, uby, M.Tp, Tb, g);
+    nee_mass(c, cf, cb, M.ux, M.uy, ubx, uby, M.Cp, Cb, h);
 }
 
 // Pre-collision populations of node (i, j) on a grid with wall nodes: the plain pull

@@ -6,6 +6,7 @@
 
 #include "lbm_kernels.cuh"
 #include "lbm_pair.cuh"
+#include "lbm_trio.cuh"
 
 namespace lbm {
 
@@ -103,13 +104,22 @@ cudaError_t launch_step_ab(const void* src, void* dst, void* hist, const Geom& G
             return launch_pdl(k, dim3((unsigned)blocks), dim3(128), L.stream, (const S*)src, (S*)dst, (R*)hist, G, c,
                               more...);
         };
+        const long long nodes = (long long)G.nx * G.ny, ring = c.nee ? ring_count(G) : 0;
+        if (trio_fits(G, c)) {   // three warps for 32 nodes
+            const unsigned rb = (unsigned)((ring + TRIO_NODES - 1) / TRIO_NODES);
+            const unsigned ib = (unsigned)((nodes - ring + TRIO_NODES - 1) / TRIO_NODES);
+            auto* k = c.nee ? step_ab_trio_kernel<true, false>
+                            : c.moving ? step_ab_trio_kernel<false, true> : step_ab_trio_kernel<false, false>;
+            return launch_pdl(k, dim3(rb + ib), dim3(TRIO_THREADS), L.stream, (const S*)src, (S*)dst, (R*)hist, G, c,
+                              rb);
+        }
         if (c.nee) {
             const long long rb = (ring_count(G) + 127) / 128;
             const long long ib = ((long long)(G.nx - 2) * (G.ny - 2) + 127) / 128;
             return c.poro ? go(step_ab_nee_flat_kernel<true>, rb + ib, (unsigned)rb)
                           : go(step_ab_nee_flat_kernel<false>, rb + ib, (unsigned)rb);
         }
-        const long long nb = ((long long)G.nx * G.ny + 127) / 128;
+        const long long nb = (nodes + 127) / 128;
         return ext ? go(step_ab_flat_kernel<true>, nb) : go(step_ab_flat_kernel<false>, nb);
     } else {
     if constexpr (LBM_AB_NEE_FUSED) {
