@@ -609,9 +609,9 @@ lbm_status lbm_batch_create(const lbm_instance* inst, int count, int capacity, s
     if (b->stream == nullptr || b->stream == cudaStreamLegacy || b->stream == cudaStreamPerThread)
         b->graph_chunk = 0;
     switch (b->prec) {
-        case LBM_F32: b->bps = batch_step_blocks_per_sm<float>(b->layout == LBM_AA); break;
-        case LBM_BF16: b->bps = batch_step_blocks_per_sm<__nv_bfloat16>(b->layout == LBM_AA); break;
-        default: b->bps = batch_step_blocks_per_sm<__half>(b->layout == LBM_AA); break;
+        case LBM_F32: b->bps = batch_residual_blocks_per_sm<float>(b->layout == LBM_AA); break;
+        case LBM_BF16: b->bps = batch_residual_blocks_per_sm<__nv_bfloat16>(b->layout == LBM_AA); break;
+        default: b->bps = batch_residual_blocks_per_sm<__half>(b->layout == LBM_AA); break;
     }
     size_t need = 0;
     for (int k = 0; k < count; ++k)
@@ -818,9 +818,9 @@ lbm_status lbm_batch_residual(lbm_batch* b, double* r, int* diverged) {
     const int grid = reduce_grid(b);
     cudaError_t e;
     switch (b->prec) {
-        case LBM_F32: e = launch_batch_residual<float>(b->d_table, b->d_owner, b->d_ntiles, b->total_tiles, b->capacity, b->parity(), aa, grid, b->d_partial, b->d_out, b->stream); break;
-        case LBM_BF16: e = launch_batch_residual<__nv_bfloat16>(b->d_table, b->d_owner, b->d_ntiles, b->total_tiles, b->capacity, b->parity(), aa, grid, b->d_partial, b->d_out, b->stream); break;
-        default: e = launch_batch_residual<__half>(b->d_table, b->d_owner, b->d_ntiles, b->total_tiles, b->capacity, b->parity(), aa, grid, b->d_partial, b->d_out, b->stream); break;
+        case LBM_F32: e = launch_batch_residual<float>(b->d_table, b->d_owner, b->d_ntiles, b->total_tiles, b->capacity, b->parity(), aa, b->has_nee, grid, b->d_partial, b->d_out, b->stream); break;
+        case LBM_BF16: e = launch_batch_residual<__nv_bfloat16>(b->d_table, b->d_owner, b->d_ntiles, b->total_tiles, b->capacity, b->parity(), aa, b->has_nee, grid, b->d_partial, b->d_out, b->stream); break;
+        default: e = launch_batch_residual<__half>(b->d_table, b->d_owner, b->d_ntiles, b->total_tiles, b->capacity, b->parity(), aa, b->has_nee, grid, b->d_partial, b->d_out, b->stream); break;
     }
     std::vector<double> h((size_t)b->capacity * 9, 0.0);
     if (e == cudaSuccess && b->total_tiles > 0)

@@ -17,12 +17,13 @@ cudaError_t launch_batch_step(const BatchInst<float>* table, const int* owner, i
 template <typename S>
 cudaError_t launch_batch_residual(const BatchInst<float>* table, const int* owner,
                                   const int* ntiles, int total_tiles, int n_inst, int parity,
-                                  bool aa, int grid, double* partial, double* out, cudaStream_t st);
+                                  bool aa, bool nee, int grid, double* partial, double* out,
+                                  cudaStream_t st);
 template <typename S>
 cudaError_t launch_batch_nush(const BatchInst<float>* table, const WallSpec* walls, int n_inst,
                               int parity, bool aa, double* out, cudaStream_t st);
-// Resident blocks per SM of the batched step kernel.
+// Resident blocks per SM of the residual pass.
 template <typename S>
-int batch_step_blocks_per_sm(bool aa);
+int batch_residual_blocks_per_sm(bool aa);
 
 }  // namespace lbm

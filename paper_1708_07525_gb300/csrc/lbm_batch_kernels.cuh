@@ -167,9 +167,13 @@ __device__ __forceinline__ const void* batch_cur(const BatchInst<R>& I, int pari
     return aa ? I.buf[0] : I.buf[(parity + I.phase) & 1];
 }
 
-// Residual pass 1 over tiles: partial[tile][9] as in residual_kernel.
-template <typename S, bool AA>
-__global__ void __launch_bounds__(BATCH_THREADS)
+// Residual pass 1 over tiles: partial[tile][9] as in residual_kernel.  Latency-bound (a gather
+// and three barriers per tile), so batches without wall nodes take a variant without the
+// rebuild (NEE = false), held to 80 registers (the rebuild takes 170).  GB300, a residual
+// call of 96 mixed cavities (2.2 M nodes), one kernel for both / this: FP32 two-buffer 173 /
+// 88 us, in place 110 / 86 us, BF16 136 / 96 us.
+template <typename S, bool AA, bool NEE>
+__global__ void __launch_bounds__(BATCH_THREADS, NEE ? 1 : 6)
 batch_residual_kernel(const BatchInst<typename Real<S>::type>* __restrict__ table,
                       const int* __restrict__ tile_owner, int total_tiles, int parity,
                       double* __restrict__ partial) {
@@ -201,7 +205,10 @@ batch_residual_kernel(const BatchInst<typename Real<S>::type>* __restrict__ tabl
 #pragma unroll
                 for (int q = 0; q < 4; ++q) old[q] = I.snap[q * n + kk];
                 R f[9], g[5], h[5];
-                gather<true>(mode, buf, G, i, j, I.c, f, g, h);
+                if (!AA && !NEE)
+                    gather_pull<false, true, false>(buf, G, i, j, I.c, f, g, h);
+                else
+                    gather<true>(mode, buf, G, i, j, I.c, f, g, h);
                 Macro<R> M = macro(I.c, f, g, h);
                 // differences in the compute precision on the deviations (exact for
                 // close values), as lbm_residual does

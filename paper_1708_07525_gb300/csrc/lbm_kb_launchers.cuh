@@ -38,14 +38,12 @@ cudaError_t launch_batch_step(const BatchInst<float>* table, const int* owner, i
 template <typename S>
 cudaError_t launch_batch_residual(const BatchInst<float>* table, const int* owner,
                                   const int* ntiles, int total_tiles, int n_inst, int parity,
-                                  bool aa, int grid, double* partial, double* out, cudaStream_t st) {
+                                  bool aa, bool nee, int grid, double* partial, double* out,
+                                  cudaStream_t st) {
     if (total_tiles <= 0 || n_inst <= 0) return cudaSuccess;
-    if (aa)
-        batch_residual_kernel<S, true><<<grid, BATCH_THREADS, 0, st>>>(table, owner, total_tiles,
-                                                                       parity, partial);
-    else
-        batch_residual_kernel<S, false><<<grid, BATCH_THREADS, 0, st>>>(table, owner, total_tiles,
-                                                                        parity, partial);
+    auto* pass = aa ? batch_residual_kernel<S, true, false>
+                    : nee ? batch_residual_kernel<S, false, true> : batch_residual_kernel<S, false, false>;
+    pass<<<grid, BATCH_THREADS, 0, st>>>(table, owner, total_tiles, parity, partial);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     batch_residual_fold_kernel<float><<<n_inst, BATCH_THREADS, 0, st>>>(table, ntiles, partial, out);
@@ -64,12 +62,10 @@ cudaError_t launch_batch_nush(const BatchInst<float>* table, const WallSpec* wal
 }
 
 template <typename S>
-int batch_step_blocks_per_sm(bool aa) {
+int batch_residual_blocks_per_sm(bool aa) {
     int n = 0;
-    if (aa)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_step_kernel<S, true>, BATCH_THREADS, 0);
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_step_kernel<S, false>, BATCH_THREADS, 0);
+    auto* pass = aa ? batch_residual_kernel<S, true, false> : batch_residual_kernel<S, false, false>;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pass, BATCH_THREADS, 0);
     return n > 0 ? n : 1;
 }
 
@@ -77,10 +73,10 @@ int batch_step_blocks_per_sm(bool aa) {
     template cudaError_t launch_batch_step<S>(const BatchInst<float>*, const int*, int, int, int,  \
                                               bool, bool, bool, cudaStream_t);                     \
     template cudaError_t launch_batch_residual<S>(const BatchInst<float>*, const int*, const int*, \
-                                                  int, int, int, bool, int, double*, double*,      \
-                                                  cudaStream_t);                                   \
+                                                  int, int, int, bool, bool, int, double*,         \
+                                                  double*, cudaStream_t);                          \
     template cudaError_t launch_batch_nush<S>(const BatchInst<float>*, const WallSpec*, int, int,  \
                                               bool, double*, cudaStream_t);                        \
-    template int batch_step_blocks_per_sm<S>(bool);
+    template int batch_residual_blocks_per_sm<S>(bool);
 
 }  // namespace lbm
