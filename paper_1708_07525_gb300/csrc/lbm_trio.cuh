@@ -7,14 +7,17 @@
 // first warp through shared memory and u comes back (on wall nodes once more, whose rebuild
 // needs the interior node's u first).  The arithmetic is collide_fixed()'s and nee_rebuild()'s,
 // operation for operation, so the bits are those of one thread a node.
-// GB300, us per step, one thread / one warp a lattice: 33^2 7.1 / 4.8, 64^2 7.1 / 5.7, 101^2 10.2 /
-// 6.7, 128^2 12.5 / 8.4, 200^2 13.6 / 8.9, 256^2 13.8 / 13.9, 512^2 41 / 45; with wall nodes
-// 33^2 14.2 / 8.1, 101^2 15.7 / 9.2, 200^2 19.6 / 11.8, 256^2 20.4 / 14.4, 300^2 20.6 / 19.2,
-// 362^2 22.6 / 25.5.  Eq. 18 solved by each warp for itself, without the way back: 64^2 6.1,
-// 101^2 9.8, 128^2 11.4 (the FP64 pipe is the scarce unit as soon as an SM has two blocks).
+// GB300, us per step, one thread / one warp a lattice: 33^2 7.1 / 4.7, 64^2 7.1 / 5.3, 101^2 10.2 /
+// 6.8, 128^2 12.5 / 8.6, 200^2 13.6 / 8.9, 249^2 13.8 / 13.2, 512^2 41 / 45; with wall nodes 33^2
+// 14.2 / 7.9, 101^2 15.7 / 8.7, 200^2 19.6 / 11.1, 249^2 20.4 / 13.8, 300^2 20.6 / 18.3, 362^2
+// 22.6 / 25.5.  Eq. 18 solved by each warp for itself, without the way back: 64^2 6.1, 101^2
+// 9.8, 128^2 11.4 (the FP64 pipe is the scarce unit as soon as an SM has two blocks).
 // A block has a fourth warp, which leaves at once: a warp's sub-partition is its number
 // modulo 4, so that each block's first warp, which has the FP64 chain, would lie elsewhere
 // with three (101^2 7.9, 101^2 with wall nodes 10.9, elsewhere within 3 percent).
+// Both scalars run one code, since a lone warp waits for instructions as long as for its own
+// results (a code each: 64^2 5.7, 64^2 with wall nodes 8.2); seven blocks per SM (72 registers, 16
+// bytes of spills; eight: 128^2 9.0, 200^2 9.4; left at 80 registers: 200^2 11.2).
 #pragma once
 #include "lbm_kernels.cuh"
 
@@ -58,7 +61,7 @@ __device__ __forceinline__ FixedMacro trio_macro(const Coef<double>& c, int role
 // NEE: nodes on the walls (the first ring_blocks blocks take them); else MOVING: halfway walls
 // that move.  Uniform porous constants, factors that fit (c.fx.on).
 template <bool NEE, bool MOVING>
-__global__ void __launch_bounds__(TRIO_THREADS)
+__global__ void __launch_bounds__(TRIO_THREADS, 7)
 step_ab_trio_kernel(const double* __restrict__ src, double* __restrict__ dst, double* __restrict__ hist, Geom G,
                     const __grid_constant__ Coef<double> c, unsigned ring_blocks) {
     __shared__ double s_wall[4][TRIO_NODES], s_mom[4][TRIO_NODES];   // jx, jy, T', C'
@@ -147,10 +150,8 @@ step_ab_trio_kernel(const double* __restrict__ src, double* __restrict__ dst, do
         for (int q = 0; q < 9; ++q) p[(size_t)q * G.plane] = d[q];
         return;
     }
-    if (role == 1)
-        fixed_scalar(c.fx.zs, add_(c.T0, s_mom[2][lane]), M, d, v, E, s, hv, top);
-    else
-        fixed_scalar(c.fx.es, add_(c.C0, s_mom[3][lane]), M, d, v, E, s, hv, top);
+    const FixedScalar& r = role == 1 ? c.fx.zs : c.fx.es;
+    fixed_scalar(r, add_(role == 1 ? c.T0 : c.C0, s_mom[role + 1][lane]), M, d, v, E, s, hv, top);
     if (!on) return;
 #pragma unroll
     for (int q = 0; q < 5; ++q) p[(size_t)q * G.plane] = d[q];
