@@ -10,8 +10,9 @@
  * plus four history values per node (T u, C u at the previous step) for the
  * explicit time derivative in the source terms of Eq. 27.
  *
- * One time step = one fused pass over the nodes (one kernel launch, or two
- * where the outermost ring of nodes has a launch of its own): pull-streaming
+ * One time step = one fused pass over the nodes (one kernel launch; two where
+ * the outermost ring of nodes has a launch of its own; half of one in large
+ * FP32 cavities, whose launches take two steps): pull-streaming
  * (Eq. 11) with the wall rules, macroscopic fields (Eqs. 16, 18-19, 26), total
  * force (Eqs. 5-6), the D2Q9 collision in moment space (Eq. 10 with Eqs.
  * 12-15) and the two D2Q5 collisions (Eqs. 21-22 with Eqs. 24-25, 27).
@@ -93,7 +94,8 @@ typedef struct {
     int block_x, block_y;       /* launch tile of the one-step kernels: block_x a multiple of 32,
                                    block_x * block_y <= 256; 0 -> tuned default (and two
                                    steps per launch where that is faster: FP32, two buffers,
-                                   halfway walls, from 750,000 nodes on) */
+                                   halfway walls, from 750,000 nodes on).  FP64 steps of an
+                                   undivided cavity have a tile of their own */
     int graph_chunk;            /* steps per captured CUDA graph; 0 -> default, <0 -> off */
     const double* eps_field;    /* optional host [ny][nx] porosity field: the REV model with
                                    spatially varying eps (Sec. 2-3 applied per node, F_eps of
@@ -229,7 +231,9 @@ lbm_status lbm_reset(lbm_ctx* ctx, const double* T_init, const double* C_init, u
  * a step that is one kernel goes out as a programmatic dependent launch: its blocks may
  * be placed while the kernel before it on the stream drains, but each waits for that
  * kernel to complete before it touches the state, so work of the caller's on the same
- * stream, before or after, is ordered as in plain stream order. */
+ * stream, before or after, is ordered as in plain stream order.  A caller may capture
+ * fewer steps than graph_chunk into a graph of its own; with an even n the graph can be
+ * replayed (each replay takes n steps, which lbm_time does not count). */
 lbm_status lbm_step(lbm_ctx* ctx, int64_t n);
 
 /* Number of time steps taken since creation (or since the loaded checkpoint). */

@@ -244,11 +244,18 @@ struct HostSlots {
     bool taken[kSlots] = {};
     double* take() {
         std::lock_guard<std::mutex> lk(mu);
-        if (!block && cudaHostAlloc((void**)&block, sizeof(double) * kSlots * kDoubles,
-                                    cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
-            cudaGetLastError();
-            block = nullptr;
-            return nullptr;
+        if (!block) {
+            // another thread may be capturing: pinning memory does not touch its streams
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            const cudaError_t e = cudaHostAlloc((void**)&block, sizeof(double) * kSlots * kDoubles,
+                                                cudaHostAllocPortable | cudaHostAllocMapped);
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                block = nullptr;
+                return nullptr;
+            }
         }
         for (int k = 0; k < kSlots; ++k)
             if (!taken[k]) {
@@ -312,6 +319,10 @@ struct lbm_ctx {
     cudaGraphExec_t graph[2][4] = {};
     int graph_end[2][4] = {};
     int64_t launched = 0;           // steps taken by launches of their own
+    // the caller has captured steps of this context: every step is a launch from then on, so
+    // that an even number of them ends on the buffers it began with and the graph can be
+    // replayed, with or without other steps in between
+    bool caller_graph = false, stale_graphs = false;
     lbm_alloc_fn alloc = nullptr;
     lbm_free_fn free_fn = nullptr;
     void* alloc_user = nullptr;
@@ -396,7 +407,22 @@ cudaError_t one_step(lbm_ctx* c) {
 
 // Two steps in one launch (lbm_march.cuh): FP32, two buffers, halfway walls, a second
 // history buffer, which only cavities that take them have.
-bool can_march(const lbm_ctx* c) { return c->hist_alt != nullptr && !c->P.nee; }
+bool can_march(const lbm_ctx* c) { return c->hist_alt != nullptr && !c->P.nee && !c->caller_graph; }
+
+// The caller is capturing the context's stream (the legacy stream cannot be captured).
+bool captured_by_caller(const lbm_ctx* c) {
+    if (c->stream == nullptr || c->stream == cudaStreamLegacy) return false;
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(c->stream, &s) == cudaSuccess && s != cudaStreamCaptureStatusNone;
+}
+
+void drop_graphs(lbm_ctx* c) {
+    for (auto& kind : c->graph)
+        for (cudaGraphExec_t& g : kind) {
+            if (g) cudaGraphExecDestroy(g);
+            g = nullptr;
+        }
+}
 
 cudaError_t two_steps(lbm_ctx* c) {
     cudaError_t e = launch_step2_ab(c->buf[c->cur], c->buf[c->cur ^ 1], c->hist, c->hist_alt, c->G, c->cf, c->L);
@@ -963,6 +989,12 @@ lbm_status lbm_step(lbm_ctx* c, int64_t n) {
     }
     DeviceGuard dg(c->device);
     cudaError_t e = cudaSuccess;
+    const bool outer = captured_by_caller(c);
+    if (outer && can_march(c)) c->caller_graph = c->stale_graphs = true;
+    if (!outer && c->stale_graphs) {
+        drop_graphs(c);
+        c->stale_graphs = false;
+    }
     // the in-place layout replays its graph from even levels
     while (n > 0 && c->layout == LBM_AA && (c->t & 1) && e == cudaSuccess) {
         e = one_step(c);
@@ -973,7 +1005,7 @@ lbm_status lbm_step(lbm_ctx* c, int64_t n) {
     // 150 us, once a context has made 64 launches of its own)
     for (int kind = 0; kind < 2 && c->graph_chunk > 0; ++kind) {
         const int chunk = kind == 0 ? c->graph_chunk : SMALL_CHUNK;
-        if (kind == 1 && (c->launched < 64 || chunk >= c->graph_chunk)) break;
+        if (kind == 1 && (c->launched < 64 || chunk >= c->graph_chunk || outer)) break;
         while (n >= chunk && e == cudaSuccess) {
             // a chunk is captured once per pair of buffers it can start from, and may end
             // on the others
@@ -1397,11 +1429,7 @@ lbm_status lbm_load(lbm_ctx* c, const void* buf, size_t len) {
     c->cf.seed_off = (long long)(c->slab_y0 - c->G.jb) * c->G.pitch;
     c->cd.poro = (c->poro && c->rsz == 8) ? (const double*)c->poro : nullptr;
     c->cf.poro = (c->poro && c->rsz == 4) ? (const float*)c->poro : nullptr;
-    for (auto& kind : c->graph)             // constants are baked into the captured launches
-        for (cudaGraphExec_t& g : kind) {
-            if (g) cudaGraphExecDestroy(g);
-            g = nullptr;
-        }
+    drop_graphs(c);                         // constants are baked into the captured launches
     c->t = h.t;
     c->cur = slot;
     c->snap_valid = false;
@@ -1423,9 +1451,7 @@ void lbm_destroy(lbm_ctx* c) {
     if (!c) return;
     DeviceGuard dg(c->device);
     if (c->stream) cudaStreamSynchronize(c->stream);
-    for (auto& kind : c->graph)
-        for (cudaGraphExec_t g : kind)
-            if (g) cudaGraphExecDestroy(g);
+    drop_graphs(c);
     c->dfree(c->buf[0], c->state_bytes());
     c->dfree(c->buf[1], c->state_bytes());
     c->dfree(c->hist, c->hist_bytes());
