@@ -220,6 +220,13 @@ def steps_per_launch(args):
     return 2 if march else 1
 
 
+def f64_kernel(args):
+    """The kernel of the FP64 step (csrc/lbm_launchers.cuh)."""
+    if args.layout == "ab" and args.size ** 2 <= (90000 if args.walls == "nee" else 62500):
+        return "step_ab_trio_kernel (FP64)"
+    return "step_ab_nee_flat_kernel (FP64)" if args.walls == "nee" else f"step_{args.layout}_flat_kernel (FP64)"
+
+
 def step_launches(args, k):
     """Kernels launched by k time steps of the benchmark cavity: half as many where a launch
     takes two steps (steps_per_launch; an odd step is one of its own).  Every other step is
@@ -347,20 +354,17 @@ def run_ours(args):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "peak_source": f"{peak_kind} hbm_gbs",
-                     "kernel": (("step_ab_nee_flat_kernel (FP64)"
-                                 if args.precision == "f64" else
-                                 f"step_ab_nee_fused_kernel<{args.precision}> (wall ring and inner "
-                                 f"nodes in one launch)")
-                                if args.walls == "nee"
-                                else (f"step_{args.layout}_pair kernels<{args.precision}> (two "
+                     "kernel": f64_kernel(args) if args.precision == "f64" else
+                                (f"step_ab_nee_fused_kernel<{args.precision}> (wall ring and inner "
+                                 f"nodes in one launch)"
+                                 if args.walls == "nee"
+                                 else f"step_{args.layout}_pair kernels<{args.precision}> (two "
                                       f"nodes per thread; edge nodes one per thread in the "
                                       f"same launch)"
-                                      if args.precision in ("bf16", "f16")
-                                      else "step2_ab_kernel (two time steps per launch)"
-                                      if per == 2
-                                      else f"step_{args.layout}_flat_kernel (FP64)"
-                                      if args.precision == "f64"
-                                      else f"step_{args.layout}_kernel<{args.precision}>")),
+                                 if args.precision in ("bf16", "f16")
+                                 else "step2_ab_kernel (two time steps per launch)"
+                                 if per == 2
+                                 else f"step_{args.layout}_kernel<{args.precision}>"),
                      "kernel_us_per_launch": launch_ms * 1e3,
                      "time_steps_per_launch": per,
                      "algorithmic_bytes_per_node": bpn,

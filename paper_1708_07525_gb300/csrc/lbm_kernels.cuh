@@ -583,15 +583,15 @@ step_aa_kernel(S* __restrict__ buf, typename Real<S>::type* __restrict__ hist, G
 
 // FP64 steps, one thread per node in the order of storage without the padding.  A warp's
 // instruction costs the same whatever the number of its active lanes, in the FP64 pipe 64
-// clocks (see lbm_fixed.cuh), so every warp is full: 129^2 nodes are 521 warps for the GPU's
-// 608 sub-partitions, and 645 by rows.  Address arithmetic is small beside the collision,
-// so nodes at the walls need no launch of their own (a ring launch on a second stream took
-// the step of a 64^2 cavity from 7 to 10 us with its fork and join).
-// GB300, us per step, the collision in FP64 with the ring apart / this: 64^2 13.1 / 7.2, 256^2
-// 39.2 / 14.4, 1024^2 505 / 154, 2048^2 1992 / 581; in place 1024^2 505 / 161; 101^2 with wall
-// nodes 23.6 / 16.  Bound by latency and issue (3,100 instructions per node, 49 % issue; FP64
-// pipe 53 % busy, against 83 % before).  4 blocks of 128 threads per SM (128 registers, 120
-// bytes of spills); 3 blocks (152 registers): 1024^2 165, 2048^2 633; 5 (96): 160, 603.
+// clocks (see lbm_fixed.cuh), so every warp is full.  Address arithmetic is small beside
+// the collision, so nodes at the walls need no launch of their own (a ring launch on a second
+// stream took the step of a 64^2 cavity from 7 to 10 us with its fork and join).  The
+// two-buffer step of small cavities is in lbm_trio.cuh.
+// GB300, us per step, the collision in FP64 with the ring apart / this: 64^2 13.1 / 7.1, 256^2
+// 39.2 / 13.8, 1024^2 505 / 147, 2048^2 1992 / 567; in place 1024^2 505 / 161; 101^2 with wall
+// nodes 23.6 / 15.7.  Bound by latency and issue (2,930 instructions per node, 48 % issue; FP64
+// pipe 55 % busy, against 83 % before).  4 blocks of 128 threads per SM (128 registers); 3
+// blocks (152 registers) took 7 to 9 percent more, 5 (96) 4 percent.
 constexpr int FLAT_MIN_BLOCKS = 4;
 
 template <bool EXT>
