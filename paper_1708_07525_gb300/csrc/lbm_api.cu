@@ -319,9 +319,9 @@ struct lbm_ctx {
     cudaGraphExec_t graph[2][4] = {};
     int graph_end[2][4] = {};
     int64_t launched = 0;           // steps taken by launches of their own
-    // the caller has captured steps of this context: every step is a launch from then on, so
-    // that an even number of them ends on the buffers it began with and the graph can be
-    // replayed, with or without other steps in between
+    // the caller has captured steps (or a reset) of this context: every step is a launch from
+    // then on, so that an even number of them ends on the buffers it began with and the graph
+    // can be replayed, with or without other steps, a reset or a load in between
     bool caller_graph = false, stale_graphs = false;
     lbm_alloc_fn alloc = nullptr;
     lbm_free_fn free_fn = nullptr;
@@ -416,6 +416,18 @@ bool captured_by_caller(const lbm_ctx* c) {
     return cudaStreamIsCapturing(c->stream, &s) == cudaSuccess && s != cudaStreamCaptureStatusNone;
 }
 
+// Notes a call that is being captured.
+void note_capture(lbm_ctx* c, bool outer) {
+    if (outer && can_march(c)) c->caller_graph = c->stale_graphs = true;
+}
+
+// The buffer for a state of level t that replaces the present one: the one in which a run of
+// single steps would hold it, so that launches which the caller has captured find it.  (t
+// mod 2, until two steps per launch have swapped the buffers an odd number of times.)
+int slot_for(const lbm_ctx* c, int64_t t) {
+    return c->layout == LBM_AB_PULL ? c->cur ^ (int)((c->t ^ t) & 1) : 0;
+}
+
 void drop_graphs(lbm_ctx* c) {
     for (auto& kind : c->graph)
         for (cudaGraphExec_t& g : kind) {
@@ -453,12 +465,13 @@ cudaError_t enqueue(lbm_ctx* c, int64_t n) {
 #define LBM_DISPATCH(c, CALL_D, CALL_F, CALL_B, CALL_H) \
     ((c)->prec == LBM_F64 ? (CALL_D) : (c)->prec == LBM_F32 ? (CALL_F) : (c)->prec == LBM_BF16 ? (CALL_B) : (CALL_H))
 
-cudaError_t run_init(lbm_ctx* c, const InitSpec& I) {
+cudaError_t run_init(lbm_ctx* c, const InitSpec& I, int slot) {
     const bool pull = c->layout == LBM_AB_PULL;
-    return LBM_DISPATCH(c, launch_init<double>(c->buf[0], c->hist, c->G, c->cd, I, pull, c->stream),
-                        launch_init<float>(c->buf[0], c->hist, c->G, c->cf, I, pull, c->stream),
-                        launch_init<__nv_bfloat16>(c->buf[0], c->hist, c->G, c->cf, I, pull, c->stream),
-                        launch_init<__half>(c->buf[0], c->hist, c->G, c->cf, I, pull, c->stream));
+    void* b = c->buf[slot];
+    return LBM_DISPATCH(c, launch_init<double>(b, c->hist, c->G, c->cd, I, pull, c->stream),
+                        launch_init<float>(b, c->hist, c->G, c->cf, I, pull, c->stream),
+                        launch_init<__nv_bfloat16>(b, c->hist, c->G, c->cf, I, pull, c->stream),
+                        launch_init<__half>(b, c->hist, c->G, c->cf, I, pull, c->stream));
 }
 
 const void* cur_buf(const lbm_ctx* c) { return c->layout == LBM_AB_PULL ? c->buf[c->cur] : c->buf[0]; }
@@ -504,10 +517,12 @@ lbm_status do_init(lbm_ctx* c, const double* T_host, const double* C_host, uint6
         I.T_init = c->d_stage;
         I.C_init = c->d_stage + n;
     }
-    if (e == cudaSuccess) e = run_init(c, I);
+    note_capture(c, captured_by_caller(c));
+    const int slot = slot_for(c, 0);
+    if (e == cudaSuccess) e = run_init(c, I, slot);
     if (e != cudaSuccess) return c->cuda_fail(e, "init");
     c->t = 0;
-    c->cur = 0;
+    c->cur = slot;
     c->snap_valid = false;
     return LBM_OK;
 }
@@ -990,7 +1005,7 @@ lbm_status lbm_step(lbm_ctx* c, int64_t n) {
     DeviceGuard dg(c->device);
     cudaError_t e = cudaSuccess;
     const bool outer = captured_by_caller(c);
-    if (outer && can_march(c)) c->caller_graph = c->stale_graphs = true;
+    note_capture(c, outer);
     if (!outer && c->stale_graphs) {
         drop_graphs(c);
         c->stale_graphs = false;
@@ -1375,8 +1390,7 @@ lbm_status lbm_load(lbm_ctx* c, const void* buf, size_t len) {
     if (h.pitch < h.nx || len < sizeof h + src_state + src_hist)
         return c->fail(LBM_ERR_INVALID, "lbm_load: truncated checkpoint");
     DeviceGuard dg(c->device);
-    // the two-buffer layout starts again in buffer (t mod 2)
-    const int slot = c->layout == LBM_AB_PULL ? (int)(h.t & 1) : 0;
+    const int slot = slot_for(c, h.t);
     const char* p = (const char*)buf + sizeof h;
     cudaError_t e;
     if (h.prec == c->prec && h.pitch == c->G.pitch) {
