@@ -233,7 +233,10 @@ lbm_status lbm_reset(lbm_ctx* ctx, const double* T_init, const double* C_init, u
  * kernel to complete before it touches the state, so work of the caller's on the same
  * stream, before or after, is ordered as in plain stream order.  A caller may capture
  * fewer steps than graph_chunk into a graph of its own; with an even n the graph can be
- * replayed (each replay takes n steps, which lbm_time does not count). */
+ * replayed (each replay takes n steps, which lbm_time does not count), also after other
+ * steps, lbm_reset or lbm_load have brought the context to a level of the parity it was
+ * captured at.  Where a launch takes two steps (lbm_options, block_x), a context that has been
+ * captured takes n mod 4 of the steps of a call one by one instead of n mod 2. */
 lbm_status lbm_step(lbm_ctx* ctx, int64_t n);
 
 /* Number of time steps taken since creation (or since the loaded checkpoint). */

@@ -319,9 +319,10 @@ struct lbm_ctx {
     cudaGraphExec_t graph[2][4] = {};
     int graph_end[2][4] = {};
     int64_t launched = 0;           // steps taken by launches of their own
-    // the caller has captured steps (or a reset) of this context: every step is a launch from
-    // then on, so that an even number of them ends on the buffers it began with and the graph
-    // can be replayed, with or without other steps, a reset or a load in between
+    // the caller has captured steps (or a reset) of this context: from then on every call and
+    // chunk takes an even number of two-step launches, so that an even number of steps ends on
+    // the buffers it began with and the graph can be replayed, with or without other steps, a
+    // reset or a load in between
     bool caller_graph = false, stale_graphs = false;
     lbm_alloc_fn alloc = nullptr;
     lbm_free_fn free_fn = nullptr;
@@ -407,7 +408,7 @@ cudaError_t one_step(lbm_ctx* c) {
 
 // Two steps in one launch (lbm_march.cuh): FP32, two buffers, halfway walls, a second
 // history buffer, which only cavities that take them have.
-bool can_march(const lbm_ctx* c) { return c->hist_alt != nullptr && !c->P.nee && !c->caller_graph; }
+bool can_march(const lbm_ctx* c) { return c->hist_alt != nullptr && !c->P.nee; }
 
 // The caller is capturing the context's stream (the legacy stream cannot be captured).
 bool captured_by_caller(const lbm_ctx* c) {
@@ -418,7 +419,7 @@ bool captured_by_caller(const lbm_ctx* c) {
 
 // Notes a call that is being captured.
 void note_capture(lbm_ctx* c, bool outer) {
-    if (outer && can_march(c)) c->caller_graph = c->stale_graphs = true;
+    if (outer && can_march(c) && !c->caller_graph) c->caller_graph = c->stale_graphs = true;
 }
 
 // The buffer for a state of level t that replaces the present one: the one in which a run of
@@ -448,17 +449,11 @@ cudaError_t two_steps(lbm_ctx* c) {
 // Enqueues n steps; stops at the first error.
 cudaError_t enqueue(lbm_ctx* c, int64_t n) {
     cudaError_t e = cudaSuccess;
-    const bool march = can_march(c);
     c->launched += n;
-    while (n > 0 && e == cudaSuccess) {
-        if (march && n >= 2) {
-            e = two_steps(c);
-            n -= 2;
-        } else {
-            e = one_step(c);
-            n -= 1;
-        }
-    }
+    // n mod 4 single steps instead of n mod 2 keep the number of two-step launches even
+    int64_t pairs = !can_march(c) ? 0 : c->caller_graph ? n / 4 * 2 : n / 2;
+    for (n -= 2 * pairs; pairs > 0 && e == cudaSuccess; --pairs) e = two_steps(c);
+    for (; n > 0 && e == cudaSuccess; --n) e = one_step(c);
     return e;
 }
 
