@@ -212,14 +212,6 @@ def run_reference(args):
     return 0
 
 
-def steps_per_launch(args):
-    """Two time steps per launch for the FP32 two-buffer cavity with halfway walls from
-    750,000 nodes on (csrc/lbm_march.cuh; not with a launch tile given), else one."""
-    march = (args.precision == "f32" and args.layout == "ab" and args.walls == "halfway"
-             and args.size ** 2 >= 750000 and not args.bx and not args.by)
-    return 2 if march else 1
-
-
 def f64_kernel(args):
     """The kernel of the FP64 step (csrc/lbm_launchers.cuh)."""
     if args.layout == "ab" and args.size ** 2 <= (90000 if args.walls == "nee" else 62500):
@@ -227,11 +219,10 @@ def f64_kernel(args):
     return "step_ab_nee_flat_kernel (FP64)" if args.walls == "nee" else f"step_{args.layout}_flat_kernel (FP64)"
 
 
-def step_launches(args, k):
-    """Kernels launched by k time steps of the benchmark cavity: half as many where a launch
-    takes two steps (steps_per_launch; an odd step is one of its own).  Every other step is
-    one launch, walls included, in every precision and layout."""
-    per = steps_per_launch(args)
+def step_launches(per, k):
+    """Kernels launched by k time steps of the benchmark cavity, of which a launch takes `per`
+    (Cavity.steps_per_launch: 2 or 1; an odd step is a launch of its own).  Walls are part of
+    the launch in every precision and layout."""
     return k // per + k % per
 
 
@@ -329,7 +320,7 @@ def run_ours(args):
 
     peak, peak_kind = measured_peaks()
     # a launch reads the state once and writes it once, whatever the steps it takes
-    per = steps_per_launch(args)
+    per = cav.steps_per_launch()
     launch_ms = kernel_ms * per
     bpn = BYTES_PER_NODE[args.precision]
     achieved = nodes * bpn / (launch_ms / 1e3) / 1e9
@@ -372,7 +363,7 @@ def run_ours(args):
                          nodes * BYTES_PER_NODE_19[args.precision] / (launch_ms / 1e3) / 1e9 / peak},
         "e2e": {"value": e2e_value, "unit": "GLUPS",
                 "h2d_bytes_per_step": 2 * nodes * 8, "d2h_bytes_per_step": 4 * 8},
-        "gpu_launches": args.steps * (step_launches(args, k) + 1 + 1),   # + Nu/Sh + residual
+        "gpu_launches": args.steps * (step_launches(per, k) + 1 + 1),   # + Nu/Sh + residual
         "clocks": clk.summary(),
         "nusselt_sherwood": [float(x) for x in nush],
     }

@@ -242,6 +242,11 @@ lbm_status lbm_step(lbm_ctx* ctx, int64_t n);
 /* Number of time steps taken since creation (or since the loaded checkpoint). */
 int64_t lbm_time(const lbm_ctx* ctx);
 
+/* Time steps that a launch of lbm_step takes: 2 where the context takes two at a time (see
+ * lbm_options, block_x; the steps of a call that are left over are launches of their own),
+ * else 1.  0 for NULL. */
+int lbm_steps_per_launch(const lbm_ctx* ctx);
+
 /* Macroscopic fields at the current time level, before collision:
  * u from Eq. 18, T and C from Eq. 26, rho from Eq. 16.  Caller-owned host
  * arrays [ny][nx]; any pointer may be NULL.  Synchronises the stream. */

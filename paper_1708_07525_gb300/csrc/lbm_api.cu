@@ -1066,6 +1066,8 @@ lbm_status lbm_step(lbm_ctx* c, int64_t n) {
 
 int64_t lbm_time(const lbm_ctx* c) { return c ? c->t : -1; }
 
+int lbm_steps_per_launch(const lbm_ctx* c) { return !c ? 0 : can_march(c) ? 2 : 1; }
+
 lbm_status lbm_fields_window(lbm_ctx* c, int x0, int y0, int w, int h, double* ux, double* uy,
                              double* T, double* C, double* rho) {
     if (!c) {

@@ -95,6 +95,8 @@ def lib():
             L.lbm_step.argtypes = [P, C.c_int64]
             L.lbm_time.argtypes = [P]
             L.lbm_time.restype = C.c_int64
+            L.lbm_steps_per_launch.argtypes = [P]
+            L.lbm_steps_per_launch.restype = C.c_int
             L.lbm_fields.argtypes = [P, dp, dp, dp, dp, dp]
             L.lbm_fields_window.argtypes = [P, C.c_int, C.c_int, C.c_int, C.c_int, dp, dp, dp, dp, dp]
             L.lbm_nusselt_sherwood.argtypes = [P, dp]
@@ -286,6 +288,10 @@ class Cavity:
     @property
     def t(self) -> int:
         return int(lib().lbm_time(self.h))
+
+    def steps_per_launch(self) -> int:
+        """lbm_steps_per_launch: the time steps that a launch takes (2 or 1)."""
+        return int(lib().lbm_steps_per_launch(self.h))
 
     def reset(self, T_init=None, C_init=None, seed=1, noise=1e-3, T_ptr=None, C_ptr=None):
         """Back to t = 0 from host fields (numpy arrays, or raw host pointers T_ptr /
