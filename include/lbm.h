@@ -94,8 +94,9 @@ typedef struct {
     int block_x, block_y;       /* launch tile of the one-step kernels: block_x a multiple of 32,
                                    block_x * block_y <= 256; 0 -> tuned default (and two
                                    steps per launch where that is faster: FP32, two buffers,
-                                   halfway walls, from 750,000 nodes on).  FP64 steps of an
-                                   undivided cavity have a tile of their own */
+                                   halfway walls, from 750,000 nodes on; see
+                                   lbm_steps_per_launch).  FP64 steps of an undivided
+                                   cavity have a tile of their own */
     int graph_chunk;            /* steps per captured CUDA graph; 0 -> default, <0 -> off */
     const double* eps_field;    /* optional host [ny][nx] porosity field: the REV model with
                                    spatially varying eps (Sec. 2-3 applied per node, F_eps of

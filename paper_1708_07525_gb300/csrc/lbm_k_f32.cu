@@ -6,9 +6,16 @@ namespace lbm {
 
 // Whether a cavity takes two steps per launch: its two buffers and history no longer stay in
 // the 126 MB L2 between steps (168 bytes per node; the measurements stand in lbm_march.cuh),
-// and the state's byte offsets fit 32 bits.
+// the state's byte offsets fit 32 bits, and strips and bands do not repeat too much of it.
+// A band of n rows stages 2 (ceil(n / 2) + 1): with fewer than 6 rows, or 7, that is more than
+// 1.4 n (us per step, two / one per launch, 760,000 nodes: 3 rows 30.6 / 19.8, 4 22.3 / 19.8,
+// 5 24.0 / 19.9, 6 19.1 / 19.8, 7 21.5 / 19.7, 8 19.6 / 19.8, 9 19.0 / 19.9; 3 million: 4 rows
+// 83 / 82, 5 86 / 81, 6 69 / 81, 7 75 / 82).  Rows of 32 columns are two strips, but one warp
+// and whole lines to the one-step kernel (65,535 rows: 66.5 / 57.5; 31 columns 69.4 / 90.1,
+// 33 columns 76.0 / 113).
 bool march_fits(const Geom& G) {
-    return (long long)G.nx * G.ny >= 750000 && (unsigned long long)(NQ + 1) * G.plane * 4 < (1ull << 32);
+    return (long long)G.nx * G.ny >= 750000 && (unsigned long long)(NQ + 1) * G.plane * 4 < (1ull << 32) &&
+           10LL * ((G.ny + 1) / 2 + 1) <= 7LL * G.ny && G.nx != 32;
 }
 
 // Rows per band: the even number up to 32 for which the last wave of warps wastes least, a
