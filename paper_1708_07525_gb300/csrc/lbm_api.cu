@@ -863,8 +863,8 @@ lbm_status create_core(const lbm_params* params, const lbm_options* opt, int sla
     c->buf[0] = c->dalloc(c->state_bytes());
     if (c->layout == LBM_AB_PULL) c->buf[1] = c->dalloc(c->state_bytes());
     c->hist = c->dalloc(c->hist_bytes());
-    if (c->prec == LBM_F32 && c->layout == LBM_AB_PULL && !slab && !O.eps_field && !O.K_field && !O.block_x &&
-        !O.block_y && march_fits(c->G)) {
+    if (c->prec == LBM_F32 && c->layout == LBM_AB_PULL && !c->P.nee && !slab && !O.eps_field && !O.K_field &&
+        !O.block_x && !O.block_y && march_fits(c->G)) {
         // two steps per launch write a second history buffer; without it (no memory for it, or
         // a state of more than a quarter of the device, which leaves the rest to the
         // caller) every step is a launch
