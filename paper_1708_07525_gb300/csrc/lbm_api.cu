@@ -278,9 +278,10 @@ struct HostSlots {
 HostSlots g_host_slots;
 
 // d_out: Nu/Sh of the side walls at 0, residual maxima at 8, Nu/Sh of bottom and top at
-// 20, scratch of the Nu/Sh pass at 64.
+// 20, scratch of the Nu/Sh pass at 64, behind it the slots of the residual pass.  Both are
+// zero at create, and every pass leaves them so.
 constexpr int SMALL_CHUNK = 8;      // steps of the smaller captured chunk (even)
-constexpr int OUT_SCRATCH = 64, OUT_DOUBLES = OUT_SCRATCH + NUSH_SCRATCH;
+constexpr int OUT_SCRATCH = 64, OUT_SLOTS = OUT_SCRATCH + NUSH_SCRATCH, OUT_DOUBLES = OUT_SLOTS + RES_SCRATCH;
 
 struct lbm_ctx {
     lbm_params P;
@@ -291,12 +292,11 @@ struct lbm_ctx {
     void* hist = nullptr;           // history of the current level
     void* hist_alt = nullptr;       // second history buffer (two steps per launch), or NULL
     int hcur = 0;                   // swaps of hist and hist_alt so far, mod 2
-    double* d_out = nullptr;        // OUT_DOUBLES: Nu/Sh and residual results, Nu/Sh partial sums
+    double* d_out = nullptr;        // OUT_DOUBLES: Nu/Sh and residual results, the passes' scratch
     double* h_out = nullptr;        // HostSlots::kDoubles of pinned memory laid out as d_out, or NULL
     double* d_fields = nullptr;     // lazily allocated [5][h][w] read-out window
     size_t fields_cap = 0;          // nodes d_fields holds
     void* d_snap = nullptr;         // lazily allocated [4][ny][nx] in the compute precision
-    double* d_partial = nullptr;    // lazily allocated residual partials
     double* d_stage = nullptr;      // lazily allocated [2][ny][nx] initial-field staging
     void* poro = nullptr;           // optional [2][ny][pitch] (eps, K) in the compute precision
     bool snap_valid = false;
@@ -936,7 +936,9 @@ lbm_status create_core(const lbm_params* params, const lbm_options* opt, int sla
     if (c->buf[1]) cudaMemsetAsync(c->buf[1], 0, c->state_bytes(), c->stream);
     cudaMemsetAsync(c->hist, 0, c->hist_bytes(), c->stream);
     if (c->hist_alt) cudaMemsetAsync(c->hist_alt, 0, c->hist_bytes(), c->stream);
-    cudaMemsetAsync(c->d_out, 0, OUT_DOUBLES * sizeof(double), c->stream);   // the block count of the Nu/Sh pass
+    // the block counts of the Nu/Sh and residual passes; here, where the stream is waited for, and
+    // not at the first read-out, which may be refused for a stream that is being captured
+    cudaMemsetAsync(c->d_out, 0, OUT_DOUBLES * sizeof(double), c->stream);
 
     if ((O.T_init == nullptr) != (O.C_init == nullptr)) {
         lbm_status s = c->fail(LBM_ERR_INVALID, "lbm_create: give both T_init and C_init");
@@ -1197,20 +1199,16 @@ lbm_status residual_maxima(lbm_ctx* c, const char* who, double h[9]) {
     const size_t n = c->nodes();
     if (!c->d_snap) {
         c->d_snap = c->dalloc(4 * n * c->rsz);
-        c->d_partial = (double*)c->dalloc(RES_SCRATCH * sizeof(double));
-        if (!c->d_snap || !c->d_partial) return c->fail(LBM_ERR_NOMEM, "%s: no device memory", who);
-        // every pass leaves its slots cleared for the next
-        const cudaError_t e = cudaMemsetAsync(c->d_partial, 0, RES_SCRATCH * sizeof(double), c->stream);
-        if (e != cudaSuccess) return c->cuda_fail(e, who);
+        if (!c->d_snap) return c->fail(LBM_ERR_NOMEM, "%s: no device memory", who);
     }
     const int mode = c->read_mode();
     const void* b = cur_buf(c);
-    double* o = out_at(c, 8);
+    double *o = out_at(c, 8), *slots = c->d_out + OUT_SLOTS;
     cudaError_t e = LBM_DISPATCH(
-        c, launch_residual<double>(b, c->G, c->cd, mode, c->d_snap, c->d_partial, o, c->stream),
-        launch_residual<float>(b, c->G, c->cf, mode, c->d_snap, c->d_partial, o, c->stream),
-        launch_residual<__nv_bfloat16>(b, c->G, c->cf, mode, c->d_snap, c->d_partial, o, c->stream),
-        launch_residual<__half>(b, c->G, c->cf, mode, c->d_snap, c->d_partial, o, c->stream));
+        c, launch_residual<double>(b, c->G, c->cd, mode, c->d_snap, slots, o, c->stream),
+        launch_residual<float>(b, c->G, c->cf, mode, c->d_snap, slots, o, c->stream),
+        launch_residual<__nv_bfloat16>(b, c->G, c->cf, mode, c->d_snap, slots, o, c->stream),
+        launch_residual<__half>(b, c->G, c->cf, mode, c->d_snap, slots, o, c->stream));
     e = fetch(c, e, 8, 9, h);
     if (e != cudaSuccess) return c->cuda_fail(e, who);
     if (h[8] != 0.0) return c->fail(LBM_ERR_DIVERGED, "%s: non-finite field at t=%lld", who, (long long)c->t);
@@ -1471,7 +1469,6 @@ void lbm_destroy(lbm_ctx* c) {
     g_host_slots.give(c->h_out);
     c->dfree(c->d_fields, 5 * c->fields_cap * sizeof(double));
     c->dfree(c->d_snap, 4 * c->nodes() * c->rsz);
-    c->dfree(c->d_partial, RES_SCRATCH * sizeof(double));
     c->dfree(c->d_stage, 2 * c->nodes() * sizeof(double));
     c->dfree(c->poro, 2 * c->G.plane * c->rsz);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);

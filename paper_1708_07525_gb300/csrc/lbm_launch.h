@@ -111,11 +111,11 @@ template <typename S>
 cudaError_t launch_nush_tb(const void* buf, const Geom& G, const Coef<typename Real<S>::type>& c,
                            int mode, const WallSpec& W, double* scratch, double* out, cudaStream_t st);
 // snap holds 4 * nx * ny values of the compute precision (FP64 for FP64 storage,
-// else FP32); partial must hold RES_SCRATCH doubles, zero at the first call and left zero by
+// else FP32); slots must hold RES_SCRATCH doubles, zero at the first call and left zero by
 // each; out 9 doubles.
 template <typename S>
 cudaError_t launch_residual(const void* buf, const Geom& G, const Coef<typename Real<S>::type>& c,
-                            int mode, void* snap, double* partial, double* out,
+                            int mode, void* snap, double* slots, double* out,
                             cudaStream_t st);
 // Copies the five populations of `row` that cross a horizontal cut moving up (up = 1)
 // or down between the state and face[5][nx] (pack = 1: state -> face).

@@ -284,10 +284,10 @@ cudaError_t launch_nush_tb(const void* buf, const Geom& G, const Coef<typename R
 
 template <typename S>
 cudaError_t launch_residual(const void* buf, const Geom& G, const Coef<typename Real<S>::type>& c,
-                            int mode, void* snap, double* partial, double* out,
+                            int mode, void* snap, double* slots, double* out,
                             cudaStream_t st) {
     using R = typename Real<S>::type;
-    return launch_residual_pass<S, R>((const S*)buf, G, c, mode, (R*)snap, partial, out, st);
+    return launch_residual_pass<S, R>((const S*)buf, G, c, mode, (R*)snap, slots, out, st);
 }
 
 template <typename S>
