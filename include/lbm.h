@@ -480,7 +480,8 @@ lbm_status lbm_server_info(const lbm_server* s, int* queued, int* active, int* d
 void lbm_server_destroy(lbm_server* s);
 const char* lbm_server_last_error(const lbm_server* s);
 
-/* Slots of 9 doubles in the fixed scratch of lbm_residual_noalloc(). */
+/* Bound of an earlier lbm_residual_noalloc(); any grid fits now.  Kept for callers that
+ * mention it. */
 #define LBM_NOALLOC_MAX_BLOCKS 4096
 
 /* The steady-state residual of lbm_residual(), for callers that cannot let the
@@ -494,17 +495,10 @@ const char* lbm_server_last_error(const lbm_server* s);
  *                  with the current fields.
  *   have_snapshot  0 if snapshot holds no earlier fields (then *r = +inf).
  *   r              host output, defined as in lbm_residual().
- * Allocates nothing: the per-block maxima are folded into one file-scope
- * device array of LBM_NOALLOC_MAX_BLOCKS * 9 + 16 doubles (about 288 KiB), which
- * every GPU that loads the library holds until the process exits; any grid fits
- * (the blocks of the first pass share its slots).  The first call on each
- * device looks up the array's device address and keeps it for the life of the
- * process (a device reset, which unloads the library's device code, makes it
- * stale); make that first call before any stream capture.  The call runs on the
- * context's device whatever device the calling thread has current.  All calls
- * share the array: each call clears it, then folds
- * into it; calls whose work overlaps on the GPU, from any context or stream,
- * race on it.  Synchronises the context's stream.  Errors as for
+ * Allocates nothing: the per-block maxima are folded into slots that the context has
+ * held since its creation, so calls on different contexts may overlap, whatever their
+ * streams and host threads.  The call runs on the context's device whatever device the
+ * calling thread has current.  Synchronises the context's stream.  Errors as for
  * lbm_residual(), plus LBM_ERR_INVALID for NULL arguments. */
 lbm_status lbm_residual_noalloc(lbm_ctx* ctx, double* snapshot, int have_snapshot, double* r);
 

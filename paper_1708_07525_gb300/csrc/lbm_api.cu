@@ -534,7 +534,9 @@ bool lbm_ctx_view(const lbm_ctx* c, CtxView* v) {
     v->mode = c->read_mode();
     v->stream = c->stream;
     v->device = c->device;
-    v->host_out = c->h_out ? c->h_out + 8 : nullptr;
+    v->slots = c->d_out + OUT_SLOTS;
+    v->out = out_at(c, 8);
+    v->out_on_host = c->h_out != nullptr;
     return true;
 }
 

@@ -167,7 +167,9 @@ struct CtxView {
     int mode;                // GATHER_* for the current level
     cudaStream_t stream;
     int device;
-    double* host_out;        // nine doubles of pinned memory for the residual's maxima, or NULL
+    double* slots;           // RES_SCRATCH doubles of the residual pass, zero between passes
+    double* out;             // where its nine results go: device memory or pinned host memory
+    bool out_on_host;
 };
 
 }  // namespace lbm
