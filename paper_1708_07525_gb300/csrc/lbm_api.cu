@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -234,29 +235,49 @@ const char* check_params(const lbm_params& P) {
 // Pinned host memory that kernels write a context's few read-out numbers to (32 doubles a
 // context), so that a read-out waits for its kernel and for no copy behind it: a copy of
 // 32 bytes to pageable memory took 8 of the 29 us of a call.  One block of the process
-// serves up to 256 contexts; it is taken with the first and given back with the last.
+// serves up to 256 contexts; it is taken with the first and given back with the last, as
+// whole pages of ordinary memory that are registered: 15 us for both (cudaHostAlloc and
+// cudaFreeHost take 250: a program with one cavity at a time waited 517 us for a cavity of
+// 64 x 64 and its end, 124 without the block).
 // A context without a slot copies its results as before.
 struct HostSlots {
     static constexpr int kSlots = 256, kDoubles = 32;
+    static constexpr size_t kBytes = sizeof(double) * kSlots * kDoubles;   // 64 KiB: whole pages of any size
     std::mutex mu;
     double* block = nullptr;
     int used = 0;
     bool taken[kSlots] = {};
+    // the block, or NULL; another thread may be capturing, whose streams this does not touch
+    static double* pin() {
+        void *p = std::aligned_alloc(kBytes, kBytes), *dev = nullptr;
+        if (!p) return nullptr;
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        cudaError_t e = cudaHostRegister(p, kBytes, cudaHostRegisterPortable | cudaHostRegisterMapped);
+        const bool pinned = e == cudaSuccess;
+        if (pinned) e = cudaHostGetDevicePointer(&dev, p, 0);
+        const bool usable = e == cudaSuccess && dev == p;      // kernels take the host's address
+        if (pinned && !usable) cudaHostUnregister(p);
+        if (e != cudaSuccess) cudaGetLastError();
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (!usable) {
+            std::free(p);
+            p = nullptr;
+        }
+        return (double*)p;
+    }
+    static void unpin(double* p) {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        const cudaError_t e = cudaHostUnregister(p);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e == cudaSuccess) std::free(p);                    // else the pages stay: the GPU may hold them
+        else cudaGetLastError();
+    }
     double* take() {
         std::lock_guard<std::mutex> lk(mu);
-        if (!block) {
-            // another thread may be capturing: pinning memory does not touch its streams
-            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-            cudaThreadExchangeStreamCaptureMode(&mode);
-            const cudaError_t e = cudaHostAlloc((void**)&block, sizeof(double) * kSlots * kDoubles,
-                                                cudaHostAllocPortable | cudaHostAllocMapped);
-            cudaThreadExchangeStreamCaptureMode(&mode);
-            if (e != cudaSuccess) {
-                cudaGetLastError();
-                block = nullptr;
-                return nullptr;
-            }
-        }
+        if (!block) block = pin();
+        if (!block) return nullptr;
         for (int k = 0; k < kSlots; ++k)
             if (!taken[k]) {
                 taken[k] = true;
@@ -270,7 +291,7 @@ struct HostSlots {
         std::lock_guard<std::mutex> lk(mu);
         taken[(p - block) / kDoubles] = false;
         if (--used == 0) {
-            cudaFreeHost(block);
+            unpin(block);
             block = nullptr;
         }
     }
