@@ -191,18 +191,24 @@ __device__ __forceinline__ f2 fma_(f2 a, f2 b, f2 c) { return f2(__ffma2_rn(a.v,
 __device__ __forceinline__ f2 fnma_(f2 a, f2 b, f2 c) {
     return f2(__ffma2_rn(make_float2(-a.v.x, -a.v.y), b.v, c.v));
 }
+__device__ __forceinline__ float round_up_ones(float x, float y);
+__device__ __forceinline__ f2 round_up_ones(f2 x, f2 y) {
+    return f2(make_float2(round_up_ones(x.v.x, y.v.x), round_up_ones(x.v.y, y.v.y)));
+}
 #endif
+}  // namespace lbm
+#include "lbm_roots.cuh"
+namespace lbm {
 
-// sqrt(x) and 1 / x of a normal x > 0, rounded to nearest.
+// sqrt(x) and 1 / x of a normal, finite x > 0.
 //   FP32: CUDA's root and division in the one-node kernels, which have all loads issued by
 //   the time these functions' branches come up (within one basic block the compiler
 //   put loads between the sums that they feed: a 256^2 step took 4.5 instead of 3.4 us).
-//   f2: per component, or (FLAT) without a branch for both at once by Markstein's sequences
-//   (P. Markstein, "IA-64 and Elementary Functions", 2000) from the special-function unit's
-//   approximation y: Newton steps on g ~ sqrt(x) and h ~ 1 / (2 sqrt(x)), or on y ~ 1 / x, and
-//   a last correction from the exact residual, which rounds as the exact result does.
+//   f2: per component, or (FLAT) without a branch for both at once from the special-function
+//   unit's approximation (lbm_roots.cuh): the same bits, rounded to nearest.
 //   FP64: the binomial series of (1 - e)^(-1/2) and (1 - e)^(-1) to second order in the
-//   error e of the approximation (below 2^-19): within an ulp, in 5 and 3 operations.
+//   error e of the approximation (below 2^-19): within one unit of the rounded result, in 5
+//   and 3 operations.
 __device__ __forceinline__ float rsqrt_seed(float x) { float y; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ float rcp_seed(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ double rsqrt_seed(double x) { double y; asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x)); return y; }
@@ -221,16 +227,11 @@ template <bool FLAT> __device__ __forceinline__ double rcp_pos(double x) {
 #ifdef __CUDACC__
 template <bool FLAT> __device__ __forceinline__ f2 sqrt_pos(f2 x) {
     if (!FLAT) return f2(make_float2(sqrtf(x.v.x), sqrtf(x.v.y)));
-    const f2 y = f2(make_float2(rsqrt_seed(x.v.x), rsqrt_seed(x.v.y)));
-    const f2 g = mul_(x, y), h = mul_(y, f2(0.5f)), r = fnma_(g, h, f2(0.5f));
-    const f2 g1 = fma_(g, r, g), h1 = fma_(h, r, h);
-    return fma_(fnma_(g1, g1, x), h1, g1);
+    return sqrt_from(x, f2(make_float2(rsqrt_seed(x.v.x), rsqrt_seed(x.v.y))));
 }
 template <bool FLAT> __device__ __forceinline__ f2 rcp_pos(f2 x) {
     if (!FLAT) return f2(make_float2(1.0f / x.v.x, 1.0f / x.v.y));
-    const f2 y = f2(make_float2(rcp_seed(x.v.x), rcp_seed(x.v.y)));
-    const f2 y1 = fma_(y, fnma_(x, y, f2(1.0f)), y);
-    return fma_(y1, fnma_(x, y1, f2(1.0f)), y1);
+    return rcp_from(x, f2(make_float2(rcp_seed(x.v.x), rcp_seed(x.v.y))));
 }
 #endif
 // Added to |v|^2 under the root, which is then never zero, and whose residual in Markstein's
