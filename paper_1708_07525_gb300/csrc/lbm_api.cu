@@ -864,6 +864,8 @@ lbm_status create_core(const lbm_params* params, const lbm_options* opt, int sla
     c->L.by = by;
     c->L.stream = c->stream;
     c->L.aux = nullptr;
+    c->L.sms = 152;
+    cudaDeviceGetAttribute(&c->L.sms, cudaDevAttrMultiProcessorCount, c->device);
     // 16-bit storage takes the two-nodes-per-thread kernels, except on slabs, whose rows
     // all run the one-node kernel (the same arithmetic as a one-node whole cavity)
     c->L.pair = (c->prec == LBM_BF16 || c->prec == LBM_F16) && !slab;

@@ -22,8 +22,8 @@ bool march_fits(const Geom& G) {
 // band of n rows costing n + 2.5 (one more row pair of stage A).  Longer bands measured slower
 // although they repeat less (4096^2: 48 rows 279.5, 96 rows 287 us; 2048^2: 26 rows 77, 98
 // rows 84 us): the warps of a wave drift apart over more rows of every plane.
-static int march_rows_per_band(const Geom& G, int strips) {
-    const long long resident = 152LL * MARCH_WARPS;
+static int march_rows_per_band(const Geom& G, int strips, int sms) {
+    const long long resident = (long long)sms * MARCH_WARPS;
     int best = 4;
     double cost = 0;
     for (int rows = 4; rows <= 32; rows += 2) {
@@ -40,7 +40,7 @@ static int march_rows_per_band(const Geom& G, int strips) {
 cudaError_t launch_step2_ab(const void* src, void* dst, const void* hist, void* hist_out, const Geom& G,
                             const Coef<float>& c, const LaunchCfg& L) {
     const int strips = (G.nx + MARCH_COLS - 1) / MARCH_COLS;
-    int rows = march_rows_per_band(G, strips);
+    int rows = march_rows_per_band(G, strips, L.sms);
     while ((G.ny + rows - 1) / rows > 65535) rows *= 2;
     const dim3 gr((unsigned)strips, (unsigned)((G.ny + rows - 1) / rows), 1);
     if (c.moving)

@@ -65,6 +65,7 @@ struct LaunchCfg {
     cudaEvent_t fork, join;
     // 16-bit storage: whether to take the two-nodes-per-thread kernels (lbm_pair.cuh)
     bool pair;
+    int sms;                // SMs of the context's device
 };
 
 // Stream for the ring launch of a split step (after forking from L.stream).
