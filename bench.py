@@ -36,6 +36,7 @@ KERNEL_SOURCES = ["paper_1708_07525_gb300/csrc/lbm_kernels.cuh",
                   "paper_1708_07525_gb300/csrc/lbm_device.cuh",
                   "paper_1708_07525_gb300/csrc/lbm_launchers.cuh",
                   "paper_1708_07525_gb300/csrc/lbm_march.cuh",
+                  "paper_1708_07525_gb300/csrc/lbm_roots.cuh",
                   "paper_1708_07525_gb300/csrc/lbm_fixed.cuh",
                   "paper_1708_07525_gb300/csrc/lbm_trio.cuh"]
 

@@ -7,7 +7,7 @@
 // the largest magnitude gets 57 bits), in which sums, differences and doublings are exact
 // and cost two instructions; products with the relaxation constants are 64 x 64 -> 128 bit
 // integer products; and what is not linear (Eqs. 5, 6, 18: two roots and a reciprocal; the
-// products of Eqs. 14, 15 and T u, C u) stays in FP64: 45 operations.
+// products of Eqs. 14, 15 and T u, C u) stays in FP64: 53 instructions per node (ncu).
 // Error: a population is rounded at 2^-58 of the node's largest (exact when within 2^4 of it;
 // the FP64 sums rounded at 2^-53 of their operands at every step), sums are exact, and a
 // result is rounded once, to nearest, when it goes back to FP64.  rho, T and C are

@@ -425,8 +425,10 @@ __device__ __forceinline__ void ab_node(const S* __restrict__ src, S* __restrict
 }
 
 // EXT = true for cavities with moving walls or porous fields, false otherwise.
-// INNER = true: the outermost ring of nodes is left to nee_ring_kernel (walls with
-// nodes on them), so this kernel keeps the plain pull's registers and occupancy.
+// INNER = true: the outermost ring of nodes has a launch of its own, so this kernel keeps
+// the plain pull's registers and occupancy.  It is the 16-bit step where the pair kernels
+// (lbm_pair.cuh) do not fit, and, beside nee_ring_kernel, the step with nodes on the walls
+// of cavities with more rows than step_ab_nee_fused_kernel's grid holds.
 template <typename S, bool EXT, bool INNER = false>
 __global__ void __launch_bounds__(256)
 step_ab_kernel(const S* __restrict__ src, S* __restrict__ dst,
@@ -481,11 +483,11 @@ step_ab_ring_kernel(const S* __restrict__ src, S* __restrict__ dst,
 }
 
 // ---- the fused step with wall nodes (Sec. 3.3), two-buffer pull layout ---------------
-// The inner nodes take step_ab_kernel<S, EXT, true> (the plain pull); nee_ring_node
-// takes the ring of wall nodes, k = 0 .. 2 nx + 2 (ny - 2) - 1 (bottom row, top row,
-// left column, right column): populations rebuilt by Eqs. 33-35 from the
-// post-streaming populations of x_f and x_ff (both pulled from src, which no
-// launch of this step writes), then the same collision as every node.
+// The inner nodes take the plain pull; nee_ring_node takes the ring of wall nodes,
+// k = 0 .. 2 nx + 2 (ny - 2) - 1 (bottom row, top row, left column, right column):
+// populations rebuilt by Eqs. 33-35 from the post-streaming populations of x_f and x_ff
+// (both pulled from src, which no launch of this step writes), then the same collision as
+// every node.
 template <typename S, typename R>
 __device__ __forceinline__ void nee_ring_node(const S* __restrict__ src, S* __restrict__ dst, R* __restrict__ hist,
                                               const Geom& G, const Coef<R>& c, long long k) {
@@ -942,7 +944,7 @@ __device__ __forceinline__ float warp_max(float v) {
 // Mean Nu / Sh on a pair of opposite walls (Eq. 38), FP64 sums with a fixed reduction
 // order (deterministic).  LR = true: the left and right walls, out = {Nu_L, Sh_L, Nu_R,
 // Sh_R}; false: bottom and top (W.Tw / W.Cw = {bottom, top}), out = {Nu_B, Sh_B, Nu_T, Sh_T}.
-// Grid (nush_blocks(G, LR), 2): block (b, s) takes the line positions b * NUSH_THREADS + t, plus
+// Grid (nush_blocks(positions along the wall), 2): block (b, s) takes the line positions b * NUSH_THREADS + t, plus
 // multiples of gridDim.x * NUSH_THREADS, of wall s, and the block that finishes last adds
 // the partial sums in block order.  `part` holds 2 * NUSH_MAX_BLOCKS pairs of doubles,
 // *done counts finished blocks (0 before the launch; the last block puts it back).

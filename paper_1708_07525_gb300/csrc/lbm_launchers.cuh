@@ -122,64 +122,64 @@ cudaError_t launch_step_ab(const void* src, void* dst, void* hist, const Geom& G
         const long long nb = (nodes + 127) / 128;
         return ext ? go(step_ab_flat_kernel<true>, nb) : go(step_ab_flat_kernel<false>, nb);
     } else {
-    if constexpr (LBM_AB_NEE_FUSED) {
-        if (c.nee) {
-            // the ring of wall nodes (the rebuild, Sec. 3.3) in the first block rows, the
-            // inner nodes (the plain pull) after them: one programmatic dependent launch
-            const long long threads = (long long)b.x * b.y;
-            const long long rrows = ((2LL * G.nx + 2LL * (G.ny - 2) + threads - 1) / threads + gr.x - 1) / gr.x;
-            if (gr.y + rrows <= 65535) {
-                const dim3 gf(gr.x, (unsigned)(gr.y + rrows), 1);
-                if (c.poro)
-                    return launch_pdl(step_ab_nee_fused_kernel<S, true>, gf, b, L.stream, (const S*)src, (S*)dst,
+        if constexpr (LBM_AB_NEE_FUSED) {
+            if (c.nee) {
+                // the ring of wall nodes (the rebuild, Sec. 3.3) in the first block rows, the
+                // inner nodes (the plain pull) after them: one programmatic dependent launch
+                const long long threads = (long long)b.x * b.y;
+                const long long rrows = ((2LL * G.nx + 2LL * (G.ny - 2) + threads - 1) / threads + gr.x - 1) / gr.x;
+                if (gr.y + rrows <= 65535) {
+                    const dim3 gf(gr.x, (unsigned)(gr.y + rrows), 1);
+                    if (c.poro)
+                        return launch_pdl(step_ab_nee_fused_kernel<S, true>, gf, b, L.stream, (const S*)src, (S*)dst,
+                                          (R*)hist, G, c, (int)rrows);
+                    return launch_pdl(step_ab_nee_fused_kernel<S, false>, gf, b, L.stream, (const S*)src, (S*)dst,
                                       (R*)hist, G, c, (int)rrows);
-                return launch_pdl(step_ab_nee_fused_kernel<S, false>, gf, b, L.stream, (const S*)src, (S*)dst,
-                                  (R*)hist, G, c, (int)rrows);
+                }
             }
         }
-    }
-    if (c.nee) {
-        // the ring of wall nodes: the rebuild (Sec. 3.3); inner nodes: the plain pull
-        cudaStream_t rs;
-        cudaError_t e = ring_fork(L, &rs);
-        if (e != cudaSuccess) return e;
-        const long long nring = 2LL * G.nx + 2LL * (G.ny - 2);
-        nee_ring_kernel<S><<<(unsigned)((nring + 127) / 128), 128, 0, rs>>>(
-            (const S*)src, (S*)dst, (R*)hist, G, c);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if (c.poro)
-            step_ab_kernel<S, true, true><<<gr, b, 0, L.stream>>>((const S*)src, (S*)dst, (R*)hist, G, c);
-        else
-            step_ab_kernel<S, false, true><<<gr, b, 0, L.stream>>>((const S*)src, (S*)dst, (R*)hist, G, c);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        return ring_join(L);
-    } else if (!std::is_same<S, float>::value && G.nx >= 3 && G.ny >= 3) {
-        // inner nodes with no wall logic, then the ring of outermost nodes.  GB300, 4096^2:
-        // BF16 385 -> 377 us, FP16 442 -> 410 us; the DRAM-bound FP32 step measured slower
-        // split (446 -> 460 us) and stays one kernel.
-        const bool ext = c.poro || c.moving;
-        cudaStream_t rs;
-        cudaError_t e = ring_fork(L, &rs);
-        if (e != cudaSuccess) return e;
-        const long long nring = 2LL * G.nx + 2LL * (G.ny - 2);
-        const unsigned nb = (unsigned)((nring + 127) / 128);
-        if (ext)
-            step_ab_ring_kernel<S, true><<<nb, 128, 0, rs>>>((const S*)src, (S*)dst, (R*)hist, G, c);
-        else
-            step_ab_ring_kernel<S, false><<<nb, 128, 0, rs>>>((const S*)src, (S*)dst, (R*)hist, G, c);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if (ext)
-            step_ab_kernel<S, true, true><<<gr, b, 0, L.stream>>>((const S*)src, (S*)dst, (R*)hist, G, c);
-        else
-            step_ab_kernel<S, false, true><<<gr, b, 0, L.stream>>>((const S*)src, (S*)dst, (R*)hist, G, c);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        return ring_join(L);
-    }
-    // one kernel per step: a programmatic dependent launch, so that this step's CTAs are
-    // placed while the step before drains
-    if (c.poro || c.moving)
-        return launch_pdl(step_ab_kernel<S, true>, gr, b, L.stream, (const S*)src, (S*)dst, (R*)hist, G, c);
-    return launch_pdl(step_ab_kernel<S, false>, gr, b, L.stream, (const S*)src, (S*)dst, (R*)hist, G, c);
+        if (c.nee) {
+            // the ring of wall nodes: the rebuild (Sec. 3.3); inner nodes: the plain pull
+            cudaStream_t rs;
+            cudaError_t e = ring_fork(L, &rs);
+            if (e != cudaSuccess) return e;
+            const long long nring = 2LL * G.nx + 2LL * (G.ny - 2);
+            nee_ring_kernel<S><<<(unsigned)((nring + 127) / 128), 128, 0, rs>>>(
+                (const S*)src, (S*)dst, (R*)hist, G, c);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if (c.poro)
+                step_ab_kernel<S, true, true><<<gr, b, 0, L.stream>>>((const S*)src, (S*)dst, (R*)hist, G, c);
+            else
+                step_ab_kernel<S, false, true><<<gr, b, 0, L.stream>>>((const S*)src, (S*)dst, (R*)hist, G, c);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            return ring_join(L);
+        } else if (!std::is_same<S, float>::value && G.nx >= 3 && G.ny >= 3) {
+            // inner nodes with no wall logic, then the ring of outermost nodes.  GB300, 4096^2:
+            // BF16 385 -> 377 us, FP16 442 -> 410 us; the DRAM-bound FP32 step measured slower
+            // split (446 -> 460 us) and stays one kernel.
+            const bool ext = c.poro || c.moving;
+            cudaStream_t rs;
+            cudaError_t e = ring_fork(L, &rs);
+            if (e != cudaSuccess) return e;
+            const long long nring = 2LL * G.nx + 2LL * (G.ny - 2);
+            const unsigned nb = (unsigned)((nring + 127) / 128);
+            if (ext)
+                step_ab_ring_kernel<S, true><<<nb, 128, 0, rs>>>((const S*)src, (S*)dst, (R*)hist, G, c);
+            else
+                step_ab_ring_kernel<S, false><<<nb, 128, 0, rs>>>((const S*)src, (S*)dst, (R*)hist, G, c);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if (ext)
+                step_ab_kernel<S, true, true><<<gr, b, 0, L.stream>>>((const S*)src, (S*)dst, (R*)hist, G, c);
+            else
+                step_ab_kernel<S, false, true><<<gr, b, 0, L.stream>>>((const S*)src, (S*)dst, (R*)hist, G, c);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            return ring_join(L);
+        }
+        // one kernel per step: a programmatic dependent launch, so that this step's CTAs are
+        // placed while the step before drains
+        if (c.poro || c.moving)
+            return launch_pdl(step_ab_kernel<S, true>, gr, b, L.stream, (const S*)src, (S*)dst, (R*)hist, G, c);
+        return launch_pdl(step_ab_kernel<S, false>, gr, b, L.stream, (const S*)src, (S*)dst, (R*)hist, G, c);
     }
 }
 
@@ -210,48 +210,48 @@ cudaError_t launch_step_aa(void* buf, void* hist, const Geom& G,
         if (odd) return ext ? go(step_aa_flat_kernel<true, true>) : go(step_aa_flat_kernel<true, false>);
         return ext ? go(step_aa_flat_kernel<false, true>) : go(step_aa_flat_kernel<false, false>);
     } else {
-    const long long split_min = LBM_AA_SPLIT_MIN_NODES;
-    if constexpr (LBM_AA_ODD_FUSED) {
-        if (odd && G.nx >= 3 && G.ny >= 3 && (long long)G.nx * G.ny >= split_min) {
-            // ring and inner nodes in one programmatic dependent launch (the ring's block
-            // rows first)
-            const long long threads = (long long)b.x * b.y;
-            const long long rrows = ((ring_count(G) + threads - 1) / threads + gr.x - 1) / gr.x;
-            if (gr.y + rrows <= 65535) {
-                const dim3 gf(gr.x, (unsigned)(gr.y + rrows), 1);
-                if (ext)
-                    return launch_pdl(step_aa_odd_fused_kernel<S, true>, gf, b, L.stream, (S*)buf, (R*)hist, G,
-                                      c, (int)rrows);
-                return launch_pdl(step_aa_odd_fused_kernel<S, false>, gf, b, L.stream, (S*)buf, (R*)hist, G, c,
-                                  (int)rrows);
+        const long long split_min = LBM_AA_SPLIT_MIN_NODES;
+        if constexpr (LBM_AA_ODD_FUSED) {
+            if (odd && G.nx >= 3 && G.ny >= 3 && (long long)G.nx * G.ny >= split_min) {
+                // ring and inner nodes in one programmatic dependent launch (the ring's block
+                // rows first)
+                const long long threads = (long long)b.x * b.y;
+                const long long rrows = ((ring_count(G) + threads - 1) / threads + gr.x - 1) / gr.x;
+                if (gr.y + rrows <= 65535) {
+                    const dim3 gf(gr.x, (unsigned)(gr.y + rrows), 1);
+                    if (ext)
+                        return launch_pdl(step_aa_odd_fused_kernel<S, true>, gf, b, L.stream, (S*)buf, (R*)hist, G,
+                                          c, (int)rrows);
+                    return launch_pdl(step_aa_odd_fused_kernel<S, false>, gf, b, L.stream, (S*)buf, (R*)hist, G, c,
+                                      (int)rrows);
+                }
             }
         }
-    }
-    if (odd && G.nx >= 3 && G.ny >= 3 && (long long)G.nx * G.ny >= split_min) {
-        // the ring of outermost nodes beside the inner nodes (no wall logic); the two
-        // launches touch disjoint locations
-        cudaStream_t rs;
-        cudaError_t e = ring_fork(L, &rs);
-        if (e != cudaSuccess) return e;
-        const long long nring = 2LL * G.nx + 2LL * (G.ny - 2);
-        const unsigned nb = (unsigned)((nring + 127) / 128);
-        if (ext)
-            step_aa_odd_ring_kernel<S, true><<<nb, 128, 0, rs>>>((S*)buf, (R*)hist, G, c);
-        else
-            step_aa_odd_ring_kernel<S, false><<<nb, 128, 0, rs>>>((S*)buf, (R*)hist, G, c);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if (ext)
-            step_aa_odd_inner_kernel<S, true><<<gr, b, 0, L.stream>>>((S*)buf, (R*)hist, G, c);
-        else
-            step_aa_odd_inner_kernel<S, false><<<gr, b, 0, L.stream>>>((S*)buf, (R*)hist, G, c);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        return ring_join(L);
-    }
-    // one kernel per step: a programmatic dependent launch, as in launch_step_ab
-    if (odd && ext) return launch_pdl(step_aa_kernel<S, true, true>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
-    if (odd) return launch_pdl(step_aa_kernel<S, true, false>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
-    if (ext) return launch_pdl(step_aa_kernel<S, false, true>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
-    return launch_pdl(step_aa_kernel<S, false, false>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
+        if (odd && G.nx >= 3 && G.ny >= 3 && (long long)G.nx * G.ny >= split_min) {
+            // the ring of outermost nodes beside the inner nodes (no wall logic); the two
+            // launches touch disjoint locations
+            cudaStream_t rs;
+            cudaError_t e = ring_fork(L, &rs);
+            if (e != cudaSuccess) return e;
+            const long long nring = 2LL * G.nx + 2LL * (G.ny - 2);
+            const unsigned nb = (unsigned)((nring + 127) / 128);
+            if (ext)
+                step_aa_odd_ring_kernel<S, true><<<nb, 128, 0, rs>>>((S*)buf, (R*)hist, G, c);
+            else
+                step_aa_odd_ring_kernel<S, false><<<nb, 128, 0, rs>>>((S*)buf, (R*)hist, G, c);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if (ext)
+                step_aa_odd_inner_kernel<S, true><<<gr, b, 0, L.stream>>>((S*)buf, (R*)hist, G, c);
+            else
+                step_aa_odd_inner_kernel<S, false><<<gr, b, 0, L.stream>>>((S*)buf, (R*)hist, G, c);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            return ring_join(L);
+        }
+        // one kernel per step: a programmatic dependent launch, as in launch_step_ab
+        if (odd && ext) return launch_pdl(step_aa_kernel<S, true, true>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
+        if (odd) return launch_pdl(step_aa_kernel<S, true, false>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
+        if (ext) return launch_pdl(step_aa_kernel<S, false, true>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
+        return launch_pdl(step_aa_kernel<S, false, false>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
     }
 }
 

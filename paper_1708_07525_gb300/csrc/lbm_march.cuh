@@ -11,10 +11,10 @@
 //     run takes half the launches;
 //   - both rows of a pair go through the collision as packed FP32x2 values (f2), whose
 //     operations round as the scalar ones do, so that two steps here give the bits of two
-//     steps of step_ab_kernel: 430 instructions per pair of nodes and step, against 545 per
-//     node there;
+//     steps of step_ab_kernel: 339 warp instructions per 32 nodes and step, repeated nodes
+//     and staging included, against 545 there (ncu, 2048^2);
 //   - a warp's rows come by asynchronous 16-byte copies into shared memory while it works on
-//     the pair before (54 rows of 128 bytes in 14 instructions); a block is one warp, so
+//     the pair before (46 rows of 128 bytes in 12 instructions); a block is one warp, so
 //     that there is no barrier, and row pointers are the same for all lanes.
 // 24 columns and not 30: what a warp stores is then whole 32-byte sectors (30 columns, whose
 // ends shared a sector with the next strip: 304 us per 4096^2 step, 24 columns: 277).  Four
@@ -180,8 +180,8 @@ __device__ __forceinline__ f2 march_pull(int q, const f2* p, const f2* n) {
     return v;
 }
 
-// Warps per SM the kernel is compiled for: at most 168 registers.  GB300, 4096^2, us per step:
-// 12 warps 277, 14 and 16 (128 registers, 52 bytes of spills) 299 and 347.
+// Warps per SM the kernel is compiled for: at most 168 registers (it takes 152).  GB300,
+// 4096^2, us per step: 12 warps 277, 14 and 16 (128 registers, 52 bytes of spills) 299 and 347.
 constexpr int MARCH_WARPS = 12;
 
 // Grid (strips, bands): block (s, b) is one warp; it stages the columns MARCH_COLS s - 4 .. + 31
