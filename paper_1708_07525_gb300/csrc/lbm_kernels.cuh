@@ -8,8 +8,8 @@ namespace lbm {
 
 // ---- programmatic dependent launch ----------------------------------------------------
 // A kernel launched by launch_pdl() may be scheduled while the kernel before it on the
-// same stream is still running.  pdl_trigger() at the start of every CTA lets the next
-// launch begin once all CTAs of this one have started; pdl_wait() holds a CTA until the
+// same stream is still running.  pdl_trigger() lets the next launch begin once all CTAs of
+// this one have come to it or ended (see pdl_start()); pdl_wait() holds a CTA until the
 // launch before it has completed and its writes are visible.  A kernel that waits before
 // its first access to the state, in every thread, and reads before that only what no
 // kernel writes, gives the results of ordinary stream order, and it completes only after
@@ -21,6 +21,15 @@ namespace lbm {
 #endif
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// When a step lets the next launch begin (late_start() in lbm_launchers.cuh says which and why): at
+// once, when the launch before this one has completed, or when this one has.
+enum { NEXT_AT_ONCE, NEXT_LATE, NEXT_AFTER };
+template <int NEXT>
+__device__ __forceinline__ void pdl_start() {
+    if (NEXT == NEXT_AT_ONCE) pdl_trigger();
+    pdl_wait();
+    if (NEXT == NEXT_LATE) pdl_trigger();
+}
 
 template <typename... P, typename... A>
 cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
@@ -429,14 +438,13 @@ __device__ __forceinline__ void ab_node(const S* __restrict__ src, S* __restrict
 // the plain pull's registers and occupancy.  It is the 16-bit step where the pair kernels
 // (lbm_pair.cuh) do not fit, and, beside nee_ring_kernel, the step with nodes on the walls
 // of cavities with more rows than step_ab_nee_fused_kernel's grid holds.
-template <typename S, bool EXT, bool INNER = false>
+template <typename S, bool EXT, bool INNER = false, int NEXT = NEXT_AT_ONCE>
 __global__ void __launch_bounds__(256)
 step_ab_kernel(const S* __restrict__ src, S* __restrict__ dst,
                typename Real<S>::type* __restrict__ hist, Geom G,
                Coef<typename Real<S>::type> c) {
     using R = typename Real<S>::type;
-    pdl_trigger();
-    pdl_wait();                                // launched by launch_pdl() in one-kernel steps
+    pdl_start<NEXT>();                         // launched by launch_step()
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = G.jb + blockIdx.y * blockDim.y + threadIdx.y;
     if (i >= G.nx || j >= G.je) return;
@@ -524,13 +532,12 @@ nee_ring_kernel(const S* __restrict__ src, S* __restrict__ dst,
 // The step with wall nodes as one launch: the first `rrows` block rows take the ring of
 // wall nodes (node k = (by gridDim.x + bx) * threads + t), the others the inner nodes
 // (row j = by - rrows) with the plain pull; held to the inner code's 64 registers.
-template <typename S, bool EXT>
+template <typename S, bool EXT, int NEXT = NEXT_AT_ONCE>
 __global__ void __launch_bounds__(256, 4)
 step_ab_nee_fused_kernel(const S* __restrict__ src, S* __restrict__ dst,
                          typename Real<S>::type* __restrict__ hist, Geom G,
                          Coef<typename Real<S>::type> c, int rrows) {
-    pdl_trigger();
-    pdl_wait();                                // launched by launch_pdl()
+    pdl_start<NEXT>();                         // launched by launch_step()
     if ((int)blockIdx.y < rrows) {
         const long long k = ((long long)blockIdx.y * gridDim.x + blockIdx.x) * (blockDim.x * blockDim.y) +
                             threadIdx.y * blockDim.x + threadIdx.x;
@@ -571,12 +578,11 @@ __device__ __forceinline__ void aa_node(S* __restrict__ buf, R* __restrict__ his
     store_hist(hist, G, self, hv);
 }
 
-template <typename S, bool ODD, bool EXT>
+template <typename S, bool ODD, bool EXT, int NEXT = NEXT_AT_ONCE>
 __global__ void __launch_bounds__(256)
 step_aa_kernel(S* __restrict__ buf, typename Real<S>::type* __restrict__ hist, Geom G,
                Coef<typename Real<S>::type> c) {
-    pdl_trigger();
-    pdl_wait();                                // launched by launch_pdl()
+    pdl_start<NEXT>();                         // launched by launch_step()
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     if (i >= G.nx || j >= G.ny) return;
@@ -590,8 +596,9 @@ step_aa_kernel(S* __restrict__ buf, typename Real<S>::type* __restrict__ hist, G
 // stream took the step of a 64^2 cavity from 7 to 10 us with its fork and join).  The
 // two-buffer step of small cavities is in lbm_trio.cuh.
 // GB300, us per step, the collision in FP64 with the ring apart / this: 64^2 13.1 / 7.1, 256^2
-// 39.2 / 13.8, 1024^2 505 / 147, 2048^2 1992 / 567; in place 1024^2 505 / 161; 101^2 with wall
-// nodes 23.6 / 15.7.  Bound by latency and issue (2,930 instructions per node, 48 % issue; FP64
+// 39.2 / 13.8, 1024^2 505 / 147, 2048^2 1992 / 567; in place 128^2 12.7 / 7.6, 1024^2 505 / 155; in a
+// porous field (the collision in FP64 too) 64^2 16.8 / 11.5, 128^2 17.0 / 11.7, 201 x 200 36.0 / 29.7,
+// 1024^2 605 / 503; 101^2 with wall nodes 23.6 / 15.7.  Bound by latency and issue (2,930 instructions per node, 48 % issue; FP64
 // pipe 55 % busy, against 83 % before).  4 blocks of 128 threads per SM (128 registers); 3
 // blocks (152 registers) took 7 to 9 percent more, 5 (96) 4 percent.
 constexpr int FLAT_MIN_BLOCKS = 4;
@@ -600,8 +607,7 @@ template <bool EXT>
 __global__ void __launch_bounds__(128, FLAT_MIN_BLOCKS)
 step_ab_flat_kernel(const double* __restrict__ src, double* __restrict__ dst, double* __restrict__ hist, Geom G,
                     Coef<double> c) {
-    pdl_trigger();
-    pdl_wait();                                // launched by launch_pdl()
+    pdl_start<EXT ? NEXT_AFTER : NEXT_AT_ONCE>();   // launched by launch_pdl()
     const unsigned k = blockIdx.x * 128u + threadIdx.x;
     if (k >= (unsigned)G.nx * (unsigned)G.ny) return;
     const unsigned j = k / (unsigned)G.nx;
@@ -614,8 +620,7 @@ template <bool EXT>
 __global__ void __launch_bounds__(128, FLAT_MIN_BLOCKS)
 step_ab_nee_flat_kernel(const double* __restrict__ src, double* __restrict__ dst, double* __restrict__ hist,
                         Geom G, Coef<double> c, unsigned ring_blocks) {
-    pdl_trigger();
-    pdl_wait();                                // launched by launch_pdl()
+    pdl_start<EXT ? NEXT_AFTER : NEXT_AT_ONCE>();   // launched by launch_pdl()
     int i, j;
     double f[9], g[5], h[5], hv[4];
     if (blockIdx.x < ring_blocks) {
@@ -643,8 +648,7 @@ step_ab_nee_flat_kernel(const double* __restrict__ src, double* __restrict__ dst
 template <bool ODD, bool EXT>
 __global__ void __launch_bounds__(128, FLAT_MIN_BLOCKS)
 step_aa_flat_kernel(double* __restrict__ buf, double* __restrict__ hist, Geom G, Coef<double> c) {
-    pdl_trigger();
-    pdl_wait();                                // launched by launch_pdl()
+    pdl_start<NEXT_AFTER>();                   // launched by launch_pdl()
     const unsigned k = blockIdx.x * 128u + threadIdx.x;
     if (k >= (unsigned)G.nx * (unsigned)G.ny) return;
     const unsigned j = k / (unsigned)G.nx;

@@ -14,6 +14,43 @@ inline dim3 grid_for(const Geom& G, int bx, int by) {
     return dim3((unsigned)((G.nx + bx - 1) / bx), (unsigned)((G.ny + by - 1) / by), 1);
 }
 
+// When a step lets the next launch in late (pdl_start()).  Let in at once, a launch that waits
+// for its turn lets the next in at once as well, and launches pile up until every SM is full; of
+// the last to fit, the blocks lie on the few SMs that had room left, and when its turn comes
+// those SMs have all of it to do (an FP64 cavity of 128^2 in a porous field 34 us per step, of
+// 64^2 11.7).  Let in late, one launch waits while one runs, at the price of a launch's latency.
+// That is better where a grid covers most of the SMs and the GPU holds two of it, and for some
+// kernels where one all but fills it.  Let in after its end, the next is placed on an empty
+// GPU: FP64 steps in place or in a porous field, which take long, and 16-bit steps in place by
+// one-node kernels.
+// GB300, us per step, at once / late: FP32 two buffers 64^2 1.68 / 1.74, 128^2 2.19 / 1.74, 256^2 3.45 /
+// 2.63, 257 x 200 (600 blocks) 2.92 / 3.40, with wall nodes 70 x 300 8.99 / 6.87; 16-bit pairs 129^2
+// 5.34 / 5.51, 144^2 4.91 / 4.23, 70 x 300 6.12 / 4.07, 288^2 4.87 / 4.99, 366^2 13.4 / 5.07, 374^2 (763
+// blocks) 4.97 / 5.05; FP64 (lbm_trio.cuh) 128^2 8.56 / 5.47, 70 x 300 (657 blocks) 7.08 / 7.84.  At
+// once / after: FP64 in a porous field 128^2 34.0 / 11.6, 201 x 200 38.3 / 29.6, 1024^2 503 / 504;
+// FP16 in place 103 x 301 3.97 / 2.38, 257 x 200 4.57 / 3.12, 383 x 260 4.61 / 4.07, lid 129 x 600
+// (1,200 blocks) 6.26 / 6.50.
+struct LateRule {            // in twentieths of a block of 128 threads per SM
+    int least, most;
+    int full, filled;        // and from .. to here, where a grid fills the GPU
+};
+constexpr LateRule LATE_F32{13, 70, 0, 0}, LATE_F32_AA{13, 70, 152, 160};          // 8 blocks per SM
+constexpr LateRule LATE_16BIT{13, 60, 0, 0}, LATE_16BIT_AA{13, 120, 0, 0};          // 5 to 8
+constexpr LateRule LATE_PAIR{19, 50, 95, 100}, LATE_TRIO{13, 70, 0, 0};             // 5, 7
+inline bool late_start(const LateRule& r, long long blocks, int threads, int sms) {
+    const long long n = 20 * blocks * threads, sm = 128LL * sms;
+    return (n >= r.least * sm && n <= r.most * sm) || (n >= r.full * sm && n <= r.filled * sm);
+}
+
+// A step in one launch, a programmatic dependent one, by the kernel that lets the next one in
+// at once or by the other.
+template <typename... P, typename... A>
+cudaError_t launch_step(void (*at_once)(P...), void (*late)(P...), const LateRule& r, dim3 grid, dim3 block,
+                        const LaunchCfg& L, A... args) {
+    const bool wait = late_start(r, (long long)grid.x * grid.y, (int)(block.x * block.y), L.sms);
+    return launch_pdl(wait ? late : at_once, grid, block, L.stream, args...);
+}
+
 template <typename S>
 cudaError_t launch_init(void* buf, void* hist, const Geom& G, const Coef<typename Real<S>::type>& c,
                         const InitSpec& I, bool pull, cudaStream_t st) {
@@ -78,6 +115,7 @@ cudaError_t launch_step_ab(const void* src, void* dst, void* hist, const Geom& G
                            const Coef<typename Real<S>::type>& c, const LaunchCfg& L) {
     using R = typename Real<S>::type;
     dim3 b(L.bx, L.by), gr = grid_for(G, L.bx, L.by);
+    constexpr LateRule rule = std::is_same<S, float>::value ? LATE_F32 : LATE_16BIT;
     if (G.jb != 0 || G.je != G.ny) {
         // a slab of a split cavity: the rows between its ghost rows, one launch with the
         // general pull (the ghost rows are ordinary neighbours, walls only where real)
@@ -94,7 +132,8 @@ cudaError_t launch_step_ab(const void* src, void* dst, void* hist, const Geom& G
         if (L.pair && !c.nee && !c.poro && !c.moving && pair_grid_ab(G, gp, erows))
             // inner column pairs two nodes per thread, the edge set one node per thread,
             // in one programmatic dependent launch
-            return launch_pdl(step_ab_pair_kernel<S>, gp, dim3(PAIR_BX, PAIR_BY), L.stream, (const S*)src,
+            return launch_step(step_ab_pair_kernel<S>, step_ab_pair_kernel<S, NEXT_LATE>, LATE_PAIR, gp,
+                               dim3(PAIR_BX, PAIR_BY), L, (const S*)src,
                               (S*)dst, (float*)hist, G, c, erows);
     }
     if constexpr (std::is_same<S, double>::value) {
@@ -108,10 +147,15 @@ cudaError_t launch_step_ab(const void* src, void* dst, void* hist, const Geom& G
         if (trio_fits(G, c)) {   // three warps for 32 nodes
             const unsigned rb = (unsigned)((ring + TRIO_NODES - 1) / TRIO_NODES);
             const unsigned ib = (unsigned)((nodes - ring + TRIO_NODES - 1) / TRIO_NODES);
-            auto* k = c.nee ? step_ab_trio_kernel<true, false>
-                            : c.moving ? step_ab_trio_kernel<false, true> : step_ab_trio_kernel<false, false>;
-            return launch_pdl(k, dim3(rb + ib), dim3(TRIO_THREADS), L.stream, (const S*)src, (S*)dst, (R*)hist, G, c,
-                              rb);
+            auto go3 = [&](auto* at_once, auto* late) {
+                return launch_step(at_once, late, LATE_TRIO, dim3(rb + ib), dim3(TRIO_THREADS), L,
+                                   (const S*)src, (S*)dst, (R*)hist, G, c, rb);
+            };
+            if (c.nee)
+                return go3(step_ab_trio_kernel<true, false, NEXT_AT_ONCE>, step_ab_trio_kernel<true, false, NEXT_LATE>);
+            if (c.moving)
+                return go3(step_ab_trio_kernel<false, true, NEXT_AT_ONCE>, step_ab_trio_kernel<false, true, NEXT_LATE>);
+            return go3(step_ab_trio_kernel<false, false, NEXT_AT_ONCE>, step_ab_trio_kernel<false, false, NEXT_LATE>);
         }
         if (c.nee) {
             const long long rb = (ring_count(G) + 127) / 128;
@@ -131,10 +175,12 @@ cudaError_t launch_step_ab(const void* src, void* dst, void* hist, const Geom& G
                 if (gr.y + rrows <= 65535) {
                     const dim3 gf(gr.x, (unsigned)(gr.y + rrows), 1);
                     if (c.poro)
-                        return launch_pdl(step_ab_nee_fused_kernel<S, true>, gf, b, L.stream, (const S*)src, (S*)dst,
-                                          (R*)hist, G, c, (int)rrows);
-                    return launch_pdl(step_ab_nee_fused_kernel<S, false>, gf, b, L.stream, (const S*)src, (S*)dst,
-                                      (R*)hist, G, c, (int)rrows);
+                        return launch_step(step_ab_nee_fused_kernel<S, true>,
+                                           step_ab_nee_fused_kernel<S, true, NEXT_LATE>, rule, gf, b, L,
+                                           (const S*)src, (S*)dst, (R*)hist, G, c, (int)rrows);
+                    return launch_step(step_ab_nee_fused_kernel<S, false>,
+                                       step_ab_nee_fused_kernel<S, false, NEXT_LATE>, rule, gf, b, L,
+                                       (const S*)src, (S*)dst, (R*)hist, G, c, (int)rrows);
                 }
             }
         }
@@ -178,8 +224,10 @@ cudaError_t launch_step_ab(const void* src, void* dst, void* hist, const Geom& G
         // one kernel per step: a programmatic dependent launch, so that this step's CTAs are
         // placed while the step before drains
         if (c.poro || c.moving)
-            return launch_pdl(step_ab_kernel<S, true>, gr, b, L.stream, (const S*)src, (S*)dst, (R*)hist, G, c);
-        return launch_pdl(step_ab_kernel<S, false>, gr, b, L.stream, (const S*)src, (S*)dst, (R*)hist, G, c);
+            return launch_step(step_ab_kernel<S, true>, step_ab_kernel<S, true, false, NEXT_LATE>, rule, gr, b, L,
+                               (const S*)src, (S*)dst, (R*)hist, G, c);
+        return launch_step(step_ab_kernel<S, false>, step_ab_kernel<S, false, false, NEXT_LATE>, rule, gr, b, L,
+                               (const S*)src, (S*)dst, (R*)hist, G, c);
     }
 }
 
@@ -189,6 +237,9 @@ cudaError_t launch_step_aa(void* buf, void* hist, const Geom& G,
                            const Coef<typename Real<S>::type>& c, bool odd, const LaunchCfg& L) {
     using R = typename Real<S>::type;
     dim3 b(L.bx, L.by), gr = grid_for(G, L.bx, L.by);
+    constexpr bool low = Store<S>::kLow;
+    constexpr LateRule rule = low ? LATE_16BIT_AA : LATE_F32_AA;
+    constexpr int later = low ? NEXT_AFTER : NEXT_LATE;
     const bool ext = c.poro || c.moving;
     if constexpr (Store<S>::kLow) {
         dim3 gp, ge;
@@ -196,9 +247,11 @@ cudaError_t launch_step_aa(void* buf, void* hist, const Geom& G,
         if (L.pair && !ext && pair_grid_ab(G, gp, erows) && pair_grid_aa_even(G, ge)) {
             const dim3 pb(PAIR_BX, PAIR_BY);
             if (!odd)
-                return launch_pdl(step_aa_even_pair_kernel<S>, ge, pb, L.stream, (S*)buf, (float*)hist, G,
+                return launch_step(step_aa_even_pair_kernel<S>, step_aa_even_pair_kernel<S, NEXT_LATE>, LATE_PAIR,
+                                   ge, pb, L, (S*)buf, (float*)hist, G,
                                   c);
-            return launch_pdl(step_aa_odd_pair_kernel<S>, gp, pb, L.stream, (S*)buf, (float*)hist, G,
+            return launch_step(step_aa_odd_pair_kernel<S>, step_aa_odd_pair_kernel<S, NEXT_LATE>, LATE_PAIR, gp, pb,
+                                   L, (S*)buf, (float*)hist, G,
                               c, erows);
         }
     }
@@ -248,10 +301,13 @@ cudaError_t launch_step_aa(void* buf, void* hist, const Geom& G,
             return ring_join(L);
         }
         // one kernel per step: a programmatic dependent launch, as in launch_step_ab
-        if (odd && ext) return launch_pdl(step_aa_kernel<S, true, true>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
-        if (odd) return launch_pdl(step_aa_kernel<S, true, false>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
-        if (ext) return launch_pdl(step_aa_kernel<S, false, true>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
-        return launch_pdl(step_aa_kernel<S, false, false>, gr, b, L.stream, (S*)buf, (R*)hist, G, c);
+        auto go = [&](auto* at_once, auto* late) {
+            return launch_step(at_once, late, rule, gr, b, L, (S*)buf, (R*)hist, G, c);
+        };
+        if (odd && ext) return go(step_aa_kernel<S, true, true>, step_aa_kernel<S, true, true, later>);
+        if (odd) return go(step_aa_kernel<S, true, false>, step_aa_kernel<S, true, false, later>);
+        if (ext) return go(step_aa_kernel<S, false, true>, step_aa_kernel<S, false, true, later>);
+        return go(step_aa_kernel<S, false, false>, step_aa_kernel<S, false, false, later>);
     }
 }
 

@@ -316,12 +316,11 @@ __device__ __forceinline__ bool loads_first(const Geom& G) {
 
 constexpr int PAIR_BX = LBM_PAIR_BX, PAIR_BY = LBM_PAIR_BY;
 
-template <typename S>
+template <typename S, int NEXT = NEXT_AT_ONCE>
 __global__ void __launch_bounds__(PAIR_BX * PAIR_BY, LBM_PAIR_MIN_BLOCKS)
 step_ab_pair_kernel(const S* __restrict__ src, S* __restrict__ dst, float* __restrict__ hist, Geom G,
                     Coef<float> c, int erows) {
-    pdl_trigger();
-    pdl_wait();                                // launched by launch_pdl()
+    pdl_start<NEXT>();                         // launched by launch_step()
     if ((int)blockIdx.y < erows) {
         const long long k = edge_index();
         if (k < edge_count(G)) ab_edge_node(src, dst, hist, G, c, k);
@@ -345,11 +344,10 @@ step_ab_pair_kernel(const S* __restrict__ src, S* __restrict__ dst, float* __res
 
 // In-place even step of every column pair (even nx): block (PAIR_BX, PAIR_BY) over
 // (nx / 2, ny).
-template <typename S>
+template <typename S, int NEXT = NEXT_AT_ONCE>
 __global__ void __launch_bounds__(PAIR_BX * PAIR_BY, LBM_PAIR_MIN_BLOCKS)
 step_aa_even_pair_kernel(S* __restrict__ buf, float* __restrict__ hist, Geom G, Coef<float> c) {
-    pdl_trigger();
-    pdl_wait();                                // launched by launch_pdl()
+    pdl_start<NEXT>();                         // launched by launch_step()
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     if (2 * m >= G.nx || j >= G.ny) return;
@@ -369,12 +367,11 @@ step_aa_even_pair_kernel(S* __restrict__ buf, float* __restrict__ hist, Geom G, 
 
 // In-place odd step: the edge blocks, then the inner column pairs (each thread reads and
 // writes only its own node's or pair's locations, so the two parts touch disjoint memory).
-template <typename S>
+template <typename S, int NEXT = NEXT_AT_ONCE>
 __global__ void __launch_bounds__(PAIR_BX * PAIR_BY, LBM_PAIR_MIN_BLOCKS)
 step_aa_odd_pair_kernel(S* __restrict__ buf, float* __restrict__ hist, Geom G, Coef<float> c,
                         int erows) {
-    pdl_trigger();
-    pdl_wait();                                // launched by launch_pdl()
+    pdl_start<NEXT>();                         // launched by launch_step()
     if ((int)blockIdx.y < erows) {
         const long long k = edge_index();
         if (k < edge_count(G)) aa_odd_edge_node(buf, hist, G, c, k);

@@ -12,6 +12,8 @@
 // 14.2 / 7.9, 101^2 15.7 / 8.7, 200^2 19.6 / 11.1, 249^2 20.4 / 13.8, 300^2 20.6 / 18.3, 362^2
 // 22.6 / 25.5.  Eq. 18 solved by each warp for itself, without the way back: 64^2 6.1, 101^2
 // 9.8, 128^2 11.4 (the FP64 pipe is the scarce unit as soon as an SM has two blocks).
+// With the next step let in late (late_start()), up to 532 blocks: 64^2 4.95, 101^2 5.5, 128^2 5.5;
+// with wall nodes 101^2 8.2, 128^2 8.5.
 // A block has a fourth warp, which leaves at once: a warp's sub-partition is its number
 // modulo 4, so that each block's first warp, which has the FP64 chain, would lie elsewhere
 // with three (101^2 7.9, 101^2 with wall nodes 10.9, elsewhere within 3 percent).
@@ -60,7 +62,7 @@ __device__ __forceinline__ FixedMacro trio_macro(const Coef<double>& c, int role
 
 // NEE: nodes on the walls (the first ring_blocks blocks take them); else MOVING: halfway walls
 // that move.  Uniform porous constants, factors that fit (c.fx.on).
-template <bool NEE, bool MOVING>
+template <bool NEE, bool MOVING, int NEXT>
 __global__ void __launch_bounds__(TRIO_THREADS, 7)
 step_ab_trio_kernel(const double* __restrict__ src, double* __restrict__ dst, double* __restrict__ hist, Geom G,
                     const __grid_constant__ Coef<double> c, unsigned ring_blocks) {
@@ -69,7 +71,7 @@ step_ab_trio_kernel(const double* __restrict__ src, double* __restrict__ dst, do
     __shared__ int s_top[3][TRIO_NODES];                             // the lattices' scales
     const int role = threadIdx.x / TRIO_NODES, lane = threadIdx.x % TRIO_NODES;
     const bool ring = NEE && blockIdx.x < ring_blocks;               // of the whole block
-    pdl_trigger();
+    if (NEXT == NEXT_AT_ONCE) pdl_trigger();
     if (role == 3) return;
     int i, j;
     bool on;                       // threads past the end repeat the last node and store nothing
@@ -89,7 +91,8 @@ step_ab_trio_kernel(const double* __restrict__ src, double* __restrict__ dst, do
     const size_t self = (size_t)j * G.pitch + i;
     const int q0 = role == 0 ? QF : role == 1 ? QG : QH;
     const double* wall = role == 1 ? c.wallT : c.wallC;
-    pdl_wait();                                // launched by launch_pdl()
+    pdl_wait();                                // launched by launch_step()
+    if (NEXT == NEXT_LATE) pdl_trigger();
     double d[9], hv[2];
     const size_t hk = (size_t)(role == 2 ? 2 : 0) * G.plane + self;
     if (role > 0) {
