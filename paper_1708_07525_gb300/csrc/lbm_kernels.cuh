@@ -750,8 +750,11 @@ step_aa_odd_ring_kernel(S* __restrict__ buf, typename Real<S>::type* __restrict_
 
 // The odd step as one launch: the first `rrows` block rows take the ring (node k =
 // (by gridDim.x + bx) * threads + t), the others the inner nodes (row j = by - rrows).
-// Held to the inner code's 64 registers (256 threads x 4 blocks); the ring code, which
-// alone takes 80, spills within that budget.
+// Held to the inner code's 64 registers (256 threads x 4 blocks).  FP32 cavities all take the
+// kernel that looks for moving walls and a porous field: compiled without them the ring's
+// code spills 56 bytes (with: none), and steps took 5.90 instead of 5.66 us at 450^2, 6.40
+// instead of 6.10 at 512^2 (odd and even steps on average; 1024^2 25.4 / 25.5).  16-bit storage
+// has few spills either way and is 4 to 8 percent faster without.
 template <typename S, bool EXT>
 __global__ void __launch_bounds__(256, 4)
 step_aa_odd_fused_kernel(S* __restrict__ buf, typename Real<S>::type* __restrict__ hist, Geom G,

@@ -272,10 +272,12 @@ cudaError_t launch_step_aa(void* buf, void* hist, const Geom& G,
                 const long long rrows = ((ring_count(G) + threads - 1) / threads + gr.x - 1) / gr.x;
                 if (gr.y + rrows <= 65535) {
                     const dim3 gf(gr.x, (unsigned)(gr.y + rrows), 1);
-                    if (ext)
-                        return launch_pdl(step_aa_odd_fused_kernel<S, true>, gf, b, L.stream, (S*)buf, (R*)hist, G,
-                                          c, (int)rrows);
-                    return launch_pdl(step_aa_odd_fused_kernel<S, false>, gf, b, L.stream, (S*)buf, (R*)hist, G, c,
+                    if constexpr (Store<S>::kLow) {
+                        if (!ext)
+                            return launch_pdl(step_aa_odd_fused_kernel<S, false>, gf, b, L.stream, (S*)buf, (R*)hist,
+                                              G, c, (int)rrows);
+                    }
+                    return launch_pdl(step_aa_odd_fused_kernel<S, true>, gf, b, L.stream, (S*)buf, (R*)hist, G, c,
                                       (int)rrows);
                 }
             }
