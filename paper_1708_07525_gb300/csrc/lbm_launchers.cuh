@@ -28,14 +28,15 @@ inline dim3 grid_for(const Geom& G, int bx, int by) {
 // 5.34 / 5.51, 144^2 4.91 / 4.23, 70 x 300 6.12 / 4.07, 288^2 4.87 / 4.99, 366^2 13.4 / 5.07, 374^2 (763
 // blocks) 4.97 / 5.05; FP64 (lbm_trio.cuh) 128^2 8.56 / 5.47, 70 x 300 (657 blocks) 7.08 / 7.84.  At
 // once / after: FP64 in a porous field 128^2 34.0 / 11.6, 201 x 200 38.3 / 29.6, 1024^2 503 / 504;
-// FP16 in place 103 x 301 3.97 / 2.38, 257 x 200 4.57 / 3.12, 383 x 260 4.61 / 4.07, lid 129 x 600
-// (1,200 blocks) 6.26 / 6.50.
+// FP16 in place 103 x 301 3.97 / 2.38, 257 x 200 4.57 / 3.12, 383 x 260 4.61 / 4.07, 501 x 301 (1,204
+// blocks) 12.3 / 5.9, lid 129 x 600 (1,200 blocks) 6.26 / 6.50.
 struct LateRule {            // in twentieths of a block of 128 threads per SM
     int least, most;
     int full, filled;        // and from .. to here, where a grid fills the GPU
 };
-constexpr LateRule LATE_F32{13, 70, 0, 0}, LATE_F32_AA{13, 70, 152, 160};          // 8 blocks per SM
+constexpr LateRule LATE_F32{13, 70, 0, 0};                                          // 8 blocks per SM
 constexpr LateRule LATE_16BIT{13, 60, 0, 0}, LATE_16BIT_AA{13, 120, 0, 0};          // 5 to 8
+constexpr LateRule LATE_AA_SPLIT{157, 160, 0, 0};      // even steps beside step_aa_odd_fused_kernel
 constexpr LateRule LATE_PAIR{19, 50, 95, 100}, LATE_TRIO{13, 70, 0, 0};             // 5, 7
 inline bool late_start(const LateRule& r, long long blocks, int threads, int sms) {
     const long long n = 20 * blocks * threads, sm = 128LL * sms;
@@ -238,7 +239,6 @@ cudaError_t launch_step_aa(void* buf, void* hist, const Geom& G,
     using R = typename Real<S>::type;
     dim3 b(L.bx, L.by), gr = grid_for(G, L.bx, L.by);
     constexpr bool low = Store<S>::kLow;
-    constexpr LateRule rule = low ? LATE_16BIT_AA : LATE_F32_AA;
     constexpr int later = low ? NEXT_AFTER : NEXT_LATE;
     const bool ext = c.poro || c.moving;
     if constexpr (Store<S>::kLow) {
@@ -264,15 +264,16 @@ cudaError_t launch_step_aa(void* buf, void* hist, const Geom& G,
         return ext ? go(step_aa_flat_kernel<false, true>) : go(step_aa_flat_kernel<false, false>);
     } else {
         const long long split_min = LBM_AA_SPLIT_MIN_NODES;
+        const bool split = G.nx >= 3 && G.ny >= 3 && (long long)G.nx * G.ny >= split_min;
         if constexpr (LBM_AA_ODD_FUSED) {
-            if (odd && G.nx >= 3 && G.ny >= 3 && (long long)G.nx * G.ny >= split_min) {
+            if (odd && split) {
                 // ring and inner nodes in one programmatic dependent launch (the ring's block
                 // rows first)
                 const long long threads = (long long)b.x * b.y;
                 const long long rrows = ((ring_count(G) + threads - 1) / threads + gr.x - 1) / gr.x;
                 if (gr.y + rrows <= 65535) {
                     const dim3 gf(gr.x, (unsigned)(gr.y + rrows), 1);
-                    if constexpr (Store<S>::kLow) {
+                    if constexpr (low) {
                         if (!ext)
                             return launch_pdl(step_aa_odd_fused_kernel<S, false>, gf, b, L.stream, (S*)buf, (R*)hist,
                                               G, c, (int)rrows);
@@ -282,7 +283,7 @@ cudaError_t launch_step_aa(void* buf, void* hist, const Geom& G,
                 }
             }
         }
-        if (odd && G.nx >= 3 && G.ny >= 3 && (long long)G.nx * G.ny >= split_min) {
+        if (odd && split) {
             // the ring of outermost nodes beside the inner nodes (no wall logic); the two
             // launches touch disjoint locations
             cudaStream_t rs;
@@ -303,9 +304,13 @@ cudaError_t launch_step_aa(void* buf, void* hist, const Geom& G,
             return ring_join(L);
         }
         // one kernel per step: a programmatic dependent launch, as in launch_step_ab
+        constexpr LateRule alone = low ? LATE_16BIT_AA : LATE_F32;
+        const LateRule& rule = split ? LATE_AA_SPLIT : alone;
         auto go = [&](auto* at_once, auto* late) {
             return launch_step(at_once, late, rule, gr, b, L, (S*)buf, (R*)hist, G, c);
         };
+        if (split && ext) return go(step_aa_kernel<S, false, true>, step_aa_kernel<S, false, true, NEXT_AFTER>);
+        if (split) return go(step_aa_kernel<S, false, false>, step_aa_kernel<S, false, false, NEXT_AFTER>);
         if (odd && ext) return go(step_aa_kernel<S, true, true>, step_aa_kernel<S, true, true, later>);
         if (odd) return go(step_aa_kernel<S, true, false>, step_aa_kernel<S, true, false, later>);
         if (ext) return go(step_aa_kernel<S, false, true>, step_aa_kernel<S, false, true, later>);
