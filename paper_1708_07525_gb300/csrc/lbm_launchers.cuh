@@ -24,7 +24,8 @@ inline dim3 grid_for(const Geom& G, int bx, int by) {
 // GPU: FP64 steps in place or in a porous field, which take long, and 16-bit steps in place by
 // one-node kernels.
 // GB300, us per step, at once / late: FP32 two buffers 64^2 1.68 / 1.74, 128^2 2.19 / 1.74, 256^2 3.45 /
-// 2.63, 257 x 200 (600 blocks) 2.92 / 3.40, with wall nodes 70 x 300 8.99 / 6.87; 16-bit pairs 129^2
+// 2.63, 257 x 200 (600 blocks) 2.92 / 3.40, with wall nodes 70 x 300 8.99 / 6.87; BF16 with wall nodes
+// 140 x 285 (578 blocks) 7.8 / 7.9, 140 x 300 (608) 12.2 / 8.0; 16-bit pairs 129^2
 // 5.34 / 5.51, 144^2 4.91 / 4.23, 70 x 300 6.12 / 4.07, 288^2 4.87 / 4.99, 366^2 13.4 / 5.07, 374^2 (763
 // blocks) 4.97 / 5.05; FP64 (lbm_trio.cuh) 128^2 8.56 / 5.47, 70 x 300 (657 blocks) 7.08 / 7.84.  At
 // once / after: FP64 in a porous field 128^2 34.0 / 11.6, 201 x 200 38.3 / 29.6, 1024^2 503 / 504;
@@ -32,10 +33,10 @@ inline dim3 grid_for(const Geom& G, int bx, int by) {
 // blocks) 12.3 / 5.9, lid 129 x 600 (1,200 blocks) 6.26 / 6.50.
 struct LateRule {            // in twentieths of a block of 128 threads per SM
     int least, most;
-    int full, filled;        // and from .. to here, where a grid fills the GPU
+    int full, filled;        // and from .. to here, where one grid (or two) fills the GPU
 };
 constexpr LateRule LATE_F32{13, 70, 0, 0};                                          // 8 blocks per SM
-constexpr LateRule LATE_16BIT{13, 60, 0, 0}, LATE_16BIT_AA{13, 120, 0, 0};          // 5 to 8
+constexpr LateRule LATE_16BIT{13, 60, 78, 80}, LATE_16BIT_AA{13, 120, 0, 0};        // 8, 5 to 8
 constexpr LateRule LATE_AA_SPLIT{157, 160, 0, 0};      // even steps beside step_aa_odd_fused_kernel
 constexpr LateRule LATE_PAIR{19, 50, 95, 100}, LATE_TRIO{13, 70, 0, 0};             // 5, 7
 inline bool late_start(const LateRule& r, long long blocks, int threads, int sms) {
